@@ -1,6 +1,7 @@
 """Builds the CUDA library (libdquant.so) in-tree with nvcc for sm_100a."""
 from __future__ import annotations
 
+import concurrent.futures
 import os
 import subprocess
 
@@ -21,6 +22,7 @@ _SOURCES = [
     ("dq_attention_wide.cu", []),
     ("dq_microbench.cu", []),
     ("dq_encode.cu", ["-fmad=false"]),
+    ("dq_encode_batch.cu", ["-fmad=false"]),
 ]
 _COMMON = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
            "-Xcompiler", "-fPIC", "-I", _INC, "-I", _CSRC]
@@ -39,15 +41,19 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(obj_dir, exist_ok=True)
     headers = [os.path.join(_CSRC, f) for f in os.listdir(_CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(_INC, "dq.h"))
-    objs = []
-    for src, extra in _SOURCES:
+
+    def compile_one(item):
+        src, extra = item
         s = os.path.join(_CSRC, src)
         o = os.path.join(obj_dir, src.replace(".cu", ".o"))
         if force or _newer(o, [s] + headers):
             cmd = [nvcc] + _COMMON + extra + os.environ.get("DQ_NVCC_EXTRA", "").split() + \
                   (["-Xptxas", "-v"] if verbose else []) + ["-c", s, "-o", o]
             subprocess.run(cmd, check=True)
-        objs.append(o)
+        return o
+
+    with concurrent.futures.ThreadPoolExecutor(max_workers=os.cpu_count() or 1) as pool:
+        objs = list(pool.map(compile_one, _SOURCES))
     if force or _newer(LIB_PATH, objs):
         tmp = LIB_PATH + f".{os.getpid()}.tmp"
         subprocess.run([nvcc] + _COMMON[:2] + ["-shared", "-o", tmp] + objs, check=True)

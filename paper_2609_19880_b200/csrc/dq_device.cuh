@@ -18,16 +18,25 @@ __device__ __forceinline__ void warp_fwht128(float (&v)[4], int lane) {
     v[1] = __fadd_rn(a1, a3); v[3] = __fsub_rn(a1, a3);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const bool upper = (lane & d) != 0;
+        const float sign = (lane & d) ? -1.f : 1.f;   // lower lane: v + other, upper lane: other - v, rounded once
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float other = __shfl_xor_sync(kFullMask, v[e], d);
-            v[e] = upper ? __fsub_rn(other, v[e]) : __fadd_rn(v[e], other);
-        }
+        for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(v[e], sign, __shfl_xor_sync(kFullMask, v[e], d));
     }
     const float sc = __uint_as_float(0x3DB504F3u);
 #pragma unroll
     for (int e = 0; e < 4; ++e) v[e] = __fmul_rn(v[e], sc);
+}
+
+// Largest / smallest of a warp's values (NaNs lose).
+__device__ __forceinline__ float warp_max(float x) {
+    float y;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float warp_min(float x) {
+    float y;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {

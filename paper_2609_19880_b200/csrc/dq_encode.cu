@@ -2,49 +2,11 @@
 // (Fig. 1 pipeline; Algorithm 1; Sec. 4.5 "Encoding").  Compiled with -fmad=false: every
 // floating-point operation below is a single IEEE operation in a fixed order so that the
 // records are reproducible bit for bit.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
+#include "dq_encode.cuh"
 
-#include <cstdlib>
-
-#include "dq_device.cuh"
-#include "dq_internal.h"
+using namespace dqenc;
 
 namespace {
-
-constexpr unsigned kFull = dqdev::kFullMask;
-constexpr int kN = DQ_HEAD_DIM;
-constexpr uint32_t kL = 1u << 23;  // lower bound of the rANS state interval (sigma = 32; token-wide streams always)
-
-using dqdev::bf16_bits_to_float;
-using dqdev::warp_fwht128;  // per-head Hadamard rotation (Sec. 4.2), 4 values per lane
-
-// Rotary position embedding of a head vector held 4 values per lane (element 4 lane + e), in
-// binary32 with every product and sum rounded once.  DQ_ROPE_HALF pairs element j with j + 64
-// (the partner sits in lane ^ 16), DQ_ROPE_PAIRS pairs 2j with 2j + 1 (same lane).
-// cs / sn: this position's 64 cosines / sines.
-__device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, const float* cs, const float* sn, int style) {
-    if (style == DQ_ROPE_HALF) {
-        const float4 c = *reinterpret_cast<const float4*>(cs + 4 * (lane & 15));
-        const float4 s = *reinterpret_cast<const float4*>(sn + 4 * (lane & 15));
-        const float cc[4] = {c.x, c.y, c.z, c.w}, ss[4] = {s.x, s.y, s.z, s.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float other = __shfl_xor_sync(kFull, v[e], 16);
-            // lanes 0-15 hold a: a cos - b sin; lanes 16-31 hold b: b cos + a sin
-            const float mine = __fmul_rn(v[e], cc[e]), cross = __fmul_rn(other, ss[e]);
-            v[e] = (lane < 16) ? __fsub_rn(mine, cross) : __fadd_rn(mine, cross);
-        }
-    } else {
-        const float2 c = *reinterpret_cast<const float2*>(cs + 2 * lane);
-        const float2 s = *reinterpret_cast<const float2*>(sn + 2 * lane);
-        const float a0 = v[0], b0 = v[1], a1 = v[2], b1 = v[3];
-        v[0] = __fsub_rn(__fmul_rn(a0, c.x), __fmul_rn(b0, s.x));
-        v[1] = __fadd_rn(__fmul_rn(b0, c.x), __fmul_rn(a0, s.x));
-        v[2] = __fsub_rn(__fmul_rn(a1, c.y), __fmul_rn(b1, s.y));
-        v[3] = __fadd_rn(__fmul_rn(b1, c.y), __fmul_rn(a1, s.y));
-    }
-}
 
 // ------------------------------------------------------------------ window means
 
@@ -135,246 +97,6 @@ dq_means_compute_kernel(const uint16_t* __restrict__ k, int T, int Hkv, int rota
                      s_first[task / Hkv], task % Hkv, lane);
 }
 
-// ------------------------------------------------------------------------ drift
-
-// Per-CTA copy of the table fields the encoder touches (a CTA encodes one tensor kind).
-// With the paired-symbol variant the rANS alphabet is the M^2 pairs u = a M + b: the coder's arrays
-// (rcp .. thr) and prk then hold the pair alphabet, r / R are not used.
-struct EncTable {
-    float r[DQ_MAX_LEVELS];
-    uint32_t R[DQ_MAX_LEVELS];
-    uint32_t rcp[DQ_MAX_PAIRS];    // Eq. rans Enc by reciprocal: floor(x / f) = umulhi(x, rcp) >> rsh
-    uint32_t rsh[DQ_MAX_PAIRS];
-    uint32_t bias[DQ_MAX_PAIRS];   // c (+ 255 when f = 1)
-    uint32_t cmpl[DQ_MAX_PAIRS];   // 2^p - f
-    uint32_t thr[DQ_MAX_PAIRS];    // f << (sigma - 9) = f L: renormalise while the state is not below it
-    uint2 prk[DQ_MAX_PAIRS];       // pairs: {bits of r_u, ceil(65536 r_u) << 8 | u}
-    int M, rec, mstar, budget_bits, has_mean, rotate;
-    int early_exit, sigma;         // codec variants: Drift tries its end multiplier first; bits of final state (32 / 24)
-    int pair;                      // paired symbols
-    uint32_t central;              // the all-central stream's four levels of a lane, one per byte
-};
-
-// Table of one tensor kind into shared memory (threads 0 .. DQ_MAX_PAIRS - 1 and thread 0).
-__device__ __forceinline__ void load_enc_table(EncTable& T, const DqDevTable& TK, const DqDevTable& TV,
-                                               const DqPairEnc& PK, const DqPairEnc& PV, bool is_v) {
-    const int pair = is_v ? TV.pair : TK.pair, sigma = is_v ? TV.sigma : TK.sigma;
-    const int i = threadIdx.x;
-    if (i < DQ_MAX_LEVELS) {
-        T.r[i] = is_v ? TV.r[i] : TK.r[i];
-        T.R[i] = is_v ? TV.R[i] : TK.R[i];
-    }
-    if (i < (pair ? DQ_MAX_PAIRS : DQ_MAX_LEVELS)) {
-        uint32_t aux;
-        if (pair) {
-            T.rcp[i] = is_v ? PV.enc_rcp[i] : PK.enc_rcp[i];
-            aux = is_v ? PV.enc_aux[i] : PK.enc_aux[i];
-            T.prk[i] = make_uint2(__float_as_uint(is_v ? PV.r[i] : PK.r[i]), ((is_v ? PV.R[i] : PK.R[i]) << 8) | (uint32_t)i);
-        } else {
-            T.rcp[i] = is_v ? TV.enc_rcp[i] : TK.enc_rcp[i];
-            aux = is_v ? TV.enc_aux[i] : TK.enc_aux[i];
-        }
-        T.bias[i] = aux & 1023u;
-        T.cmpl[i] = (aux >> 10) & 511u;
-        T.rsh[i] = aux >> 19;
-        T.thr[i] = (256u - ((aux >> 10) & 511u)) << (sigma - 9);
-    }
-    if (i == 0) {
-        T.M = is_v ? TV.M : TK.M; T.rec = is_v ? TV.rec : TK.rec; T.mstar = is_v ? TV.mstar : TK.mstar;
-        T.budget_bits = is_v ? TV.budget_bits : TK.budget_bits;
-        T.has_mean = is_v ? TV.has_mean : TK.has_mean; T.rotate = is_v ? TV.rotate : TK.rotate;
-        T.early_exit = is_v ? TV.early_exit : TK.early_exit; T.sigma = sigma;
-        T.pair = pair;
-        const uint32_t ms = (uint32_t)T.mstar, us = (uint32_t)(is_v ? TV.ustar : TK.ustar), M = (uint32_t)T.M;
-        T.central = pair ? (us / M) * 0x00010001u + (us % M) * 0x01000100u : ms * 0x01010101u;
-    }
-}
-
-// Function Drift of Algorithm 1 on a stream held 4 values per lane.  The bisection of
-// log2(lambda) over T = 12 steps is carried out as the geometric mean of the bracket
-// [hi * 2^-40, hi], hi = 8 (max D - min D); the code length is an integer sum of
-// ceil(65536 r_m), so the feasibility test does not depend on summation order.
-// Returns the length of the final assignment (the argmin at the bracket's upper end).
-// M is a template parameter so that the M candidate costs of a value are independent
-// instructions and the table sits in registers; the minimum keeps the lowest index among equal
-// costs, exactly as an ascending scan with a strict comparison does.
-template <int M>
-__device__ __noinline__ uint32_t drift_m(const EncTable& T, float z0, float z1, float z2, float z3, float s, float o,
-                                         uint32_t& sym_packed) {
-    const float z[4] = {z0, z1, z2, z3};
-    float tm[M], rm[M];
-    uint32_t Km[M];   // ceil(65536 r_m) << 8 | m: the minimum tree carries one word for length and index
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        tm[m] = __fmaf_rn((float)m, s, o);
-        rm[m] = T.r[m];
-        Km[m] = (T.R[m] << 8) | (uint32_t)m;
-    }
-    float D[4][M];
-    float maxD = -INFINITY, minD = INFINITY;
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            const float d = __fsub_rn(z[e], tm[m]);
-            D[e][m] = __fmul_rn(d, d);
-            maxD = fmaxf(maxD, D[e][m]);
-            minD = fminf(minD, D[e][m]);
-        }
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        maxD = fmaxf(maxD, __shfl_xor_sync(kFull, maxD, d));
-        minD = fminf(minD, __shfl_xor_sync(kFull, minD, d));
-    }
-    const uint32_t budget = (uint32_t)T.budget_bits << 16;
-    float lam_hi = __fmul_rn(8.0f, __fsub_rn(maxD, minD));
-    float lam_lo = __fmul_rn(lam_hi, 0x1p-40f);
-    uint32_t len = 0, sym[4] = {0u, 0u, 0u, 0u};
-    // Early-exit variant: when each of the 12 tests passes, the upper end walks hi <- sqrt(lo hi) twelve
-    // times with lo fixed; sweep -1 evaluates that multiplier and ends the search if its assignment fits.
-    float lam_e = lam_hi;
-    if (T.early_exit)
-        for (int i = 0; i < 12; ++i) lam_e = __fsqrt_rn(__fmul_rn(lam_lo, lam_e));
-#pragma unroll 1
-    for (int it = T.early_exit ? -1 : 0; it <= 12; ++it) {
-        const float lam = (it < 0) ? lam_e : (it < 12) ? __fsqrt_rn(__fmul_rn(lam_lo, lam_hi)) : lam_hi;
-        uint32_t cost_sum = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            float c[M];
-            uint32_t key[M];
-#pragma unroll
-            for (int m = 0; m < M; ++m) { c[m] = __fmaf_rn(lam, rm[m], D[e][m]); key[m] = Km[m]; }
-            // pairwise minimum, the left (lower index) operand wins ties
-#pragma unroll
-            for (int w = 1; w < M; w <<= 1)
-#pragma unroll
-                for (int m = 0; m + w < M; m += 2 * w)
-                    if (c[m + w] < c[m]) { c[m] = c[m + w]; key[m] = key[m + w]; }
-            sym[e] = key[0];
-            cost_sum += key[0];
-        }
-        len = __reduce_add_sync(kFull, cost_sum >> 8);   // four indices (< 16 each) stay below bit 8
-        if (it < 0) {
-            if (len <= budget) break;
-        } else if (it < 12) {
-            if (len <= budget) lam_hi = lam; else lam_lo = lam;
-        }
-    }
-    sym_packed = (sym[0] & 0xffu) | ((sym[1] & 0xffu) << 8) | ((sym[2] & 0xffu) << 16) | (sym[3] << 24);
-    return len;
-}
-
-__device__ __forceinline__ uint32_t drift(const EncTable& T, const float (&z)[4], float s, float o,
-                                          uint32_t (&sym)[4]) {
-    uint32_t packed = 0, len = 0;
-    switch (T.M) {   // uniform across the CTA
-#define DQ_DRIFT_CASE(M_) case M_: len = drift_m<M_>(T, z[0], z[1], z[2], z[3], s, o, packed); break;
-        DQ_DRIFT_CASE(2) DQ_DRIFT_CASE(3) DQ_DRIFT_CASE(4) DQ_DRIFT_CASE(5) DQ_DRIFT_CASE(6) DQ_DRIFT_CASE(7)
-        DQ_DRIFT_CASE(8) DQ_DRIFT_CASE(9) DQ_DRIFT_CASE(10) DQ_DRIFT_CASE(11) DQ_DRIFT_CASE(12) DQ_DRIFT_CASE(13)
-        DQ_DRIFT_CASE(14) DQ_DRIFT_CASE(15) DQ_DRIFT_CASE(16)
-#undef DQ_DRIFT_CASE
-        default: break;
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) sym[e] = (packed >> (8 * e)) & 0xffu;
-    return len;
-}
-
-// Drift for the paired-symbol variant: a lane's values (0, 1) and (2, 3) are two rANS symbols; each takes
-// the pair u = a M + b that minimises (D_a + D_b) + lambda r_u, the lowest u among equal costs (rows a in
-// ascending order, each reduced pairwise with the left operand winning ties, a later row replacing the best
-// only when strictly cheaper: the same winner as an ascending scan with a strict comparison).  Bracket: hi = 16 (max D - min D), D over single values as above.
-template <int M>
-__device__ __noinline__ uint32_t drift_pair_m(const EncTable& T, float z0, float z1, float z2, float z3, float s, float o,
-                                              uint32_t& sym_packed) {
-    const float z[4] = {z0, z1, z2, z3};
-    float D[4][M];
-    float maxD = -INFINITY, minD = INFINITY;
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        const float tm = __fmaf_rn((float)m, s, o);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float d = __fsub_rn(z[e], tm);
-            D[e][m] = __fmul_rn(d, d);
-            maxD = fmaxf(maxD, D[e][m]);
-            minD = fminf(minD, D[e][m]);
-        }
-    }
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        maxD = fmaxf(maxD, __shfl_xor_sync(kFull, maxD, d));
-        minD = fminf(minD, __shfl_xor_sync(kFull, minD, d));
-    }
-    const uint32_t budget = (uint32_t)T.budget_bits << 16;
-    float lam_hi = __fmul_rn(16.0f, __fsub_rn(maxD, minD));
-    float lam_lo = __fmul_rn(lam_hi, 0x1p-40f);
-    uint32_t len = 0, psym[2] = {0u, 0u};
-    float lam_e = lam_hi;
-    if (T.early_exit)
-        for (int i = 0; i < 12; ++i) lam_e = __fsqrt_rn(__fmul_rn(lam_lo, lam_e));
-#pragma unroll 1
-    for (int it = T.early_exit ? -1 : 0; it <= 12; ++it) {
-        const float lam = (it < 0) ? lam_e : (it < 12) ? __fsqrt_rn(__fmul_rn(lam_lo, lam_hi)) : lam_hi;
-        uint32_t cost_sum = 0;
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float rc[M];
-            uint32_t rkey[M];
-#pragma unroll
-            for (int a = 0; a < M; ++a) {
-                float c[M];
-                uint32_t key[M];
-#pragma unroll
-                for (int b = 0; b < M; ++b) {
-                    const uint2 e = T.prk[a * M + b];
-                    c[b] = __fmaf_rn(lam, __uint_as_float(e.x), __fadd_rn(D[2 * p][a], D[2 * p + 1][b]));
-                    key[b] = e.y;
-                }
-#pragma unroll
-                for (int w = 1; w < M; w <<= 1)
-#pragma unroll
-                    for (int b = 0; b + w < M; b += 2 * w)
-                        if (c[b + w] < c[b]) { c[b] = c[b + w]; key[b] = key[b + w]; }
-                rc[a] = c[0];
-                rkey[a] = key[0];
-            }
-#pragma unroll
-            for (int w = 1; w < M; w <<= 1)   // row winners, the left (lower a) operand wins ties
-#pragma unroll
-                for (int a = 0; a + w < M; a += 2 * w)
-                    if (rc[a + w] < rc[a]) { rc[a] = rc[a + w]; rkey[a] = rkey[a + w]; }
-            psym[p] = rkey[0];
-            cost_sum += rkey[0];
-        }
-        len = __reduce_add_sync(kFull, cost_sum >> 8);   // two pair indices (< 81 each) stay below bit 8
-        if (it < 0) {
-            if (len <= budget) break;
-        } else if (it < 12) {
-            if (len <= budget) lam_hi = lam; else lam_lo = lam;
-        }
-    }
-    const uint32_t u0 = psym[0] & 0xffu, u1 = psym[1] & 0xffu;
-    sym_packed = (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24);
-    return len;
-}
-
-__device__ __forceinline__ uint32_t drift_pair(const EncTable& T, const float (&z)[4], float s, float o,
-                                               uint32_t (&sym)[4]) {
-    uint32_t packed = 0, len = 0;
-    switch (T.M) {   // uniform across the CTA
-#define DQ_DRIFT_CASE(M_) case M_: len = drift_pair_m<M_>(T, z[0], z[1], z[2], z[3], s, o, packed); break;
-        DQ_DRIFT_CASE(2) DQ_DRIFT_CASE(3) DQ_DRIFT_CASE(4) DQ_DRIFT_CASE(5) DQ_DRIFT_CASE(6) DQ_DRIFT_CASE(7)
-        DQ_DRIFT_CASE(8) DQ_DRIFT_CASE(9)
-#undef DQ_DRIFT_CASE
-        default: break;
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) sym[e] = (packed >> (8 * e)) & 0xffu;
-    return len;
-}
-
 // ---------------------------------------------------------------------- encoder
 
 constexpr int kEncWarps = 8;
@@ -382,129 +104,54 @@ constexpr int kEncWarps = 8;
 #define DQ_STEP_ENC_WARPS 16
 #endif
 
-// Position and sequence of call token t (decode-step mode derives them from the sequence lengths).
-__device__ __forceinline__ int tok_pos(const DqEncodeArgs& a, int t) { return a.step_seq_lens ? a.step_seq_lens[t] - 1 : a.pos[t]; }
-__device__ __forceinline__ int tok_seq(const DqEncodeArgs& a, int t) { return a.step_seq_lens ? t : a.seq_id[t]; }
+// quantise_values for the table's number of levels: one call, everything inside it inlined.
+template <int M, bool PAIR>
+__device__ __noinline__ StreamQuantised quantise_m(const EncTable& T, float z0, float z1, float z2, float z3) {
+    const float z[4] = {z0, z1, z2, z3};
+    return quantise_values<M, PAIR>(T, z);
+}
+template <bool PAIR>
+__device__ __forceinline__ StreamQuantised quantise_any(const EncTable& T, const float (&z)[4]) {
+    switch (T.M) {   // uniform across the CTA
+#define DQ_LEVELS_CASE(M_) case M_: return quantise_m<M_, PAIR>(T, z[0], z[1], z[2], z[3]);
+        DQ_LEVELS_CASE(2) DQ_LEVELS_CASE(3) DQ_LEVELS_CASE(4) DQ_LEVELS_CASE(5) DQ_LEVELS_CASE(6) DQ_LEVELS_CASE(7)
+        DQ_LEVELS_CASE(8) default: break;
+    }
+    if constexpr (PAIR) {
+        return quantise_m<9, PAIR>(T, z[0], z[1], z[2], z[3]);
+    } else {
+        switch (T.M) {
+            DQ_LEVELS_CASE(9) DQ_LEVELS_CASE(10) DQ_LEVELS_CASE(11) DQ_LEVELS_CASE(12) DQ_LEVELS_CASE(13) DQ_LEVELS_CASE(14)
+            DQ_LEVELS_CASE(15) default: return quantise_m<16, PAIR>(T, z[0], z[1], z[2], z[3]);
+        }
+    }
+#undef DQ_LEVELS_CASE
+}
 
-struct StreamQuantised {
-    uint32_t hdr0;      // s fp16 | o fp16 << 16
-    uint32_t flags;     // 1: all-central fallback, 2: constant stream, 4: refit rejected
-    uint32_t sym;       // this lane's four symbols, one per byte
-};
-
-// Steps 1-6 of Algorithm 1 for the stream (token t, KV head h) by one warp: rotation (and rotary
-// embedding when asked), mean removal, min-max grid, drift, refit, fp16 metadata, second drift.
-// PAIR: the table's rANS symbols are pairs of levels (a kernel instantiation of its own, so that the
-// single-level kernels carry none of its code).
+// Steps 1-6 for the stream (token t, KV head h): rotary embedding when asked, rotation, mean removal, then the above.
 template <bool PAIR>
 __device__ __forceinline__ StreamQuantised quantise_stream(const EncTable& T, const DqEncodeArgs& a, bool is_v, int t, int h,
                                                            int lane) {
-    const int Hkv = a.Hkv;
     const uint16_t* x = static_cast<const uint16_t*>(is_v ? a.v_bf16 : a.k_bf16);
     float z[4];
-    {
-        const uint2 raw = *reinterpret_cast<const uint2*>(x + ((size_t)t * Hkv + h) * kN + 4 * lane);
-        z[0] = bf16_bits_to_float(raw.x & 0xffffu); z[1] = bf16_bits_to_float(raw.x >> 16);
-        z[2] = bf16_bits_to_float(raw.y & 0xffffu); z[3] = bf16_bits_to_float(raw.y >> 16);
-    }
+    unpack_bf16x4(*reinterpret_cast<const uint2*>(x + ((size_t)t * a.Hkv + h) * kN + 4 * lane), z);
     if (!is_v && a.rope_style)
         warp_rope128(z, lane, a.rope_cos + (size_t)tok_pos(a, t) * 64, a.rope_sin + (size_t)tok_pos(a, t) * 64, a.rope_style);
-    if (T.rotate) warp_fwht128(z, lane);
-    if (T.has_mean) {  // remove the (dequantised) windowed channel mean, Sec. 4.2
-        const int ps = tok_pos(a, t), w = ps / DQ_WINDOW_TOKENS;
-        const size_t mi = ((size_t)tok_seq(a, t) * a.max_windows + w) * Hkv + h;
-        uint32_t q4;
-        float sc;
+    uint32_t q4 = 0u;
+    float sc = 0.f;
+    if (T.has_mean) {
+        const int ps = tok_pos(a, t);
+        const size_t mi = mean_row(a, tok_seq(a, t), ps, h);
         if (a.mean_mode == DQ_MEAN_REUSE && ps % DQ_WINDOW_TOKENS == 0) {
-            // first position of a window: carry the previous window's mean forward (window 0: zero).
-            // Rows are per head, so this warp is the only writer and reader of the row in this call.
-            q4 = 0u; sc = 0.f;
-            if (w > 0) {
-                const size_t src = mi - (size_t)Hkv;
-                q4 = *reinterpret_cast<const uint32_t*>(a.mean_q + src * kN + 4 * lane);
-                sc = a.mean_scale[src];
-            }
-            *reinterpret_cast<uint32_t*>(a.mean_q + mi * kN + 4 * lane) = q4;
-            if (lane == 0) a.mean_scale[mi] = sc;
+            carry_mean(a, mi, ps, lane, q4, sc);
         } else {
             sc = a.mean_scale[mi];
             q4 = *reinterpret_cast<const uint32_t*>(a.mean_q + mi * kN + 4 * lane);
         }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float q = (float)(int)(int8_t)((q4 >> (8 * e)) & 0xffu);
-            z[e] = __fsub_rn(z[e], __fmul_rn(sc, q));
-        }
     }
-    float mx = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
-    float mn = fminf(fminf(z[0], z[1]), fminf(z[2], z[3]));
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, d));
-        mn = fminf(mn, __shfl_xor_sync(kFull, mn, d));
-    }
-
-    uint32_t sym[4];
-    __half s16 = __ushort_as_half(0), o16 = __ushort_as_half(0);
-    bool degenerate = !(mx > mn);
-    uint32_t st_fallback = 0, st_refit = 0;
-    if (!degenerate) {
-        const float o = mn;                                         // FitMinMax, Eq. (affine_token)
-        const float s = __fdiv_rn(__fsub_rn(mx, mn), (float)(T.M - 1));
-        if (PAIR) drift_pair(T, z, s, o, sym); else drift(T, z, s, o, sym);
-        // Refit: least squares of z on the symbols; binary64 sums in a fixed order
-        double sa = (double)z[0], sb = __dmul_rn((double)sym[0], (double)z[0]);
-        int sm = (int)sym[0], smm = (int)(sym[0] * sym[0]);
-#pragma unroll
-        for (int e = 1; e < 4; ++e) {
-            sa = __dadd_rn(sa, (double)z[e]);
-            sb = __dadd_rn(sb, __dmul_rn((double)sym[e], (double)z[e]));
-            sm += (int)sym[e];
-            smm += (int)(sym[e] * sym[e]);
-        }
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) {
-            sa = __dadd_rn(sa, __shfl_xor_sync(kFull, sa, d));
-            sb = __dadd_rn(sb, __shfl_xor_sync(kFull, sb, d));
-        }
-        const long long Sm = __reduce_add_sync(kFull, sm), Smm = __reduce_add_sync(kFull, smm);
-        const long long den = (long long)kN * Smm - Sm * Sm;
-        double sd = (double)s, od = (double)o;
-        if (den != 0) {
-            sd = __ddiv_rn(__dsub_rn(__dmul_rn((double)kN, sb), __dmul_rn((double)Sm, sa)), (double)den);
-            od = __ddiv_rn(__dsub_rn(sa, __dmul_rn(sd, (double)Sm)), (double)kN);
-        }
-        s16 = __double2half(sd);                                    // fp16 metadata
-        o16 = __double2half(od);
-        float sf = __half2float(s16), of = __half2float(o16);
-        if (!(isfinite(sf) && sf > 0.0f && isfinite(of))) {
-            s16 = __float2half_rn(s);
-            o16 = __float2half_rn(o);
-            sf = __half2float(s16); of = __half2float(o16);
-            st_refit = 1;
-        }
-        if (!(sf > 0.0f)) degenerate = true;
-        else {
-            const uint32_t len = PAIR ? drift_pair(T, z, sf, of, sym) : drift(T, z, sf, of, sym);   // second Drift, fp16 grid
-            if (len > ((uint32_t)T.budget_bits << 16)) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) sym[e] = (T.central >> (8 * e)) & 0xffu;
-                st_fallback = 1;
-            }
-        }
-    }
-    if (degenerate) {
-        s16 = __ushort_as_half(0);
-        o16 = __float2half_rn(mn);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) sym[e] = (T.central >> (8 * e)) & 0xffu;
-    }
-
-    StreamQuantised r;
-    r.hdr0 = (uint32_t)__half_as_ushort(s16) | ((uint32_t)__half_as_ushort(o16) << 16);
-    r.flags = st_fallback | (degenerate ? 2u : 0u) | (st_refit << 2);
-    r.sym = sym[0] | (sym[1] << 8) | (sym[2] << 16) | (sym[3] << 24);
-    return r;
+    if (T.rotate) warp_fwht128(z, lane);
+    if (T.has_mean) remove_mean(z, q4, sc);
+    return quantise_any<PAIR>(T, z);
 }
 
 // One warp per stream (token, KV head); lane l owns elements 4l .. 4l+3.  blockIdx.y selects
@@ -517,7 +164,7 @@ template <int MINB, int WARPS, bool PAIR>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
 dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ DqDevTable TV,
                  const __grid_constant__ DqPairEnc PK, const __grid_constant__ DqPairEnc PV, const DqEncodeArgs a) {
-    __shared__ EncTable T;
+    __shared__ __align__(16) EncTable T;
     __shared__ uint8_t s_bytes[WARPS][DQ_MAX_REC_BYTES];
     __shared__ __align__(4) uint8_t s_sym[WARPS][kN];
     // Decode-step mode: the kernels after this one start while it runs and take their own launch as proof
@@ -539,8 +186,10 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long wid = (long long)blockIdx.x * WARPS + wib;
     if (wid >= (long long)a.T * a.Hkv) return;
-    if (tok_pos(a, (int)(wid / a.Hkv)) < 0) return;   // decode-step mode: an empty sequence has no new token
-    const int t = (int)(wid / a.Hkv), h = (int)(wid % a.Hkv), Hkv = a.Hkv;
+    int t, h;
+    split_stream(a, wid, t, h);
+    const int Hkv = a.Hkv;
+    if (tok_pos(a, t) < 0) return;   // decode-step mode: an empty sequence has no new token
     uint8_t* cont = is_v ? a.v_cont : a.k_cont;
 
     const StreamQuantised sq = quantise_stream<PAIR>(T, a, is_v, t, h, lane);
@@ -563,13 +212,13 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
 #pragma unroll 8
     for (int j = (PAIR ? kN / 2 : kN) - 1; j >= 0; --j) {
         const uint32_t m = s_sym[wib][j];
-        const uint32_t rcp = T.rcp[m], rsh = T.rsh[m], bias = T.bias[m], cmpl = T.cmpl[m], thr = T.thr[m];
-        if (xs >= thr) {  // at most once: xs < 2^8 L <= 2^8 * (f L)
+        const uint4 en = T.enc[m];
+        if (xs >= en.y) {  // at most once: xs < 2^8 L <= 2^8 * (f L)
             if (lane == 0) asm volatile("st.shared.u8 [%0], %1;" ::"r"(bytes_addr + k), "r"(xs & 0xffu));
             ++k;
             xs >>= 8;
         }
-        xs = (__umulhi(xs, rcp) >> rsh) * cmpl + (xs + bias);
+        xs = (__umulhi(xs, en.x) >> (en.w >> 16)) * (en.w & 0xffffu) + (xs + en.z);
     }
     __syncwarp();
     asm volatile("" ::: "memory");
@@ -594,98 +243,6 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
     }
 }
 
-
-// Throughput variant for calls with many streams: a CTA of 4 warps takes 32 consecutive streams.
-// Each warp quantises 8 of them (steps 1-6 of Algorithm 1, as above) and leaves the symbols in
-// shared memory; then ONE warp entropy-codes all 32 streams at once, lane = stream, so the serial
-// rANS chain costs one instruction stream per 32 streams instead of one per stream with 32
-// redundant lanes.  Symbols are stored [position][stream] and emitted bytes [byte index][stream] so
-// that the lanes of that warp touch consecutive bytes.  Small CTAs, 8 per SM at 64 registers: the
-// other warps of a CTA idle during its rANS pass, so that pass should be a small part of a small CTA.
-#ifndef DQ_B32_MINB
-#define DQ_B32_MINB 8
-#endif
-#ifndef DQ_B32_WARPS
-#define DQ_B32_WARPS 4
-#endif
-constexpr int kB32 = 32;                 // streams per CTA
-constexpr int kB32SymStride = 36;        // bytes per position row (32 streams + pad against bank conflicts)
-constexpr int kB32Warps = DQ_B32_WARPS;
-constexpr int kB32PairMinBlocks = 4;   // paired symbols: the pair search wants 128 registers (7.9 ms against 12.5 ms at 8 CTAs per SM, config 2 prefill)
-template <int MINB, bool PAIR>
-__global__ void __launch_bounds__(kB32Warps * 32, MINB)
-dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ DqDevTable TV,
-                         const __grid_constant__ DqPairEnc PK, const __grid_constant__ DqPairEnc PV, const DqEncodeArgs a) {
-    __shared__ EncTable T;
-    __shared__ __align__(4) uint8_t s_symT[kN * kB32SymStride];
-    __shared__ uint8_t s_bytesT[DQ_MAX_REC_BYTES * kB32];
-    __shared__ uint32_t s_hdr[kB32], s_xs[kB32], s_k[kB32];
-    __shared__ unsigned long long s_rec[kB32];   // record addresses
-    dqdev::pdl_launch_dependents();
-    const bool is_v = a.do_k ? (blockIdx.y == 1) : true;
-    load_enc_table(T, TK, TV, PK, PV, is_v);
-    __syncthreads();
-    dqdev::pdl_wait_prior_grid();
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const long long total = (long long)a.T * a.Hkv;
-    const long long first = (long long)blockIdx.x * kB32;
-    const int ns = (int)min((long long)kB32, total - first);
-    uint8_t* cont = is_v ? a.v_cont : a.k_cont;
-
-    for (int i = wib; i < ns; i += kB32Warps) {   // quantise: warp w takes streams w, w + warps, ...
-        const long long wid = first + i;
-        const int t = (int)(wid / a.Hkv), h = (int)(wid % a.Hkv);
-        const StreamQuantised sq = quantise_stream<PAIR>(T, a, is_v, t, h, lane);
-        if (PAIR) {   // the lane's two pair indices u = a M + b at positions 2 lane, 2 lane + 1
-            const uint32_t M = (uint32_t)T.M;
-            s_symT[(2 * lane) * kB32SymStride + i] = (uint8_t)((sq.sym & 0xffu) * M + ((sq.sym >> 8) & 0xffu));
-            s_symT[(2 * lane + 1) * kB32SymStride + i] = (uint8_t)(((sq.sym >> 16) & 0xffu) * M + (sq.sym >> 24));
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) s_symT[(4 * lane + e) * kB32SymStride + i] = (uint8_t)(sq.sym >> (8 * e));
-        }
-        if (lane == 0) {
-            s_hdr[i] = sq.hdr0;
-            const int sl = a.slot[t];
-            s_rec[i] = (unsigned long long)(cont + (((size_t)(sl / DQ_PAGE_TOKENS) * a.Hkv + h) * DQ_PAGE_TOKENS +
-                                                    (size_t)(sl % DQ_PAGE_TOKENS)) * T.rec);
-            if (a.status) {
-                if (sq.flags & 1u) atomicAdd(a.status + 0, 1u);
-                if (sq.flags & 2u) atomicAdd(a.status + 1, 1u);
-                if (sq.flags & 4u) atomicAdd(a.status + 2, 1u);
-            }
-        }
-    }
-    __syncthreads();
-    if (wib == 0 && lane < ns) {   // rANS, Eq. (rans) Enc on symbols 127 .. 0; lane = stream
-        uint32_t xs = 1u << (T.sigma - 9), k = 0;
-#pragma unroll 4
-        for (int j = (PAIR ? kN / 2 : kN) - 1; j >= 0; --j) {
-            const uint32_t m = s_symT[j * kB32SymStride + lane];
-            const uint32_t rcp = T.rcp[m], rsh = T.rsh[m], bias = T.bias[m], cmpl = T.cmpl[m], thr = T.thr[m];
-            if (xs >= thr) {   // at most once: xs < 2^8 L <= 2^8 * (f L)
-                if (k < DQ_MAX_REC_BYTES) s_bytesT[k * kB32 + lane] = (uint8_t)xs;   // the budget test keeps k < rec - 8
-                ++k;
-                xs >>= 8;
-            }
-            xs = (__umulhi(xs, rcp) >> rsh) * cmpl + (xs + bias);
-        }
-        s_xs[lane] = xs;
-        s_k[lane] = k;
-        if (a.status) atomicMax(a.status + 3, 4u + (uint32_t)(T.sigma >> 3) + k);
-    }
-    __syncthreads();
-    const int rec = T.rec, pay = 4 + (T.sigma >> 3);
-    for (int idx = threadIdx.x; idx < ns * rec; idx += blockDim.x) {   // records out: header, state, k bytes, then zeros
-        const int si = idx / rec, i = idx - si * rec;
-        const int k = (int)s_k[si], used = min(pay + k, rec);
-        uint8_t v = 0;
-        if (i < 4) v = (uint8_t)(s_hdr[si] >> (8 * i));
-        else if (i < pay) v = (uint8_t)(s_xs[si] >> (8 * (i - 4)));
-        else if (i < used) v = s_bytesT[(k - 1 - (i - pay)) * kB32 + si];   // emitted last = read first
-        reinterpret_cast<uint8_t*>(s_rec[si])[i] = v;
-    }
-}
 
 // rANS encode of one stream by one warp (Eq. rans Enc on symbols n-1 .. 0 so that decoding runs
 // forward).  Every lane carries the same state; lane 0 records the emitted bytes (in emission
@@ -1136,7 +693,7 @@ template <bool PAIR>
 __global__ void __launch_bounds__(DQ_MAX_STREAM_HEADS * 32)
 dq_encode_wide_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ DqDevTable TV,
                       const __grid_constant__ DqPairEnc PK, const __grid_constant__ DqPairEnc PV, const DqEncodeArgs a) {
-    __shared__ EncTable T;
+    __shared__ __align__(16) EncTable T;
     __shared__ __align__(16) WideShared W;
     __shared__ uint8_t s_bytes[DQ_MAX_WIDE_REC_BYTES];
     __shared__ __align__(4) uint8_t s_sym[DQ_MAX_STREAM_HEADS * kN];
@@ -1179,7 +736,7 @@ __global__ void __launch_bounds__(DQ_MAX_STREAM_HEADS * 32, PAIR ? 2 : DQ_ENCW_M
 dq_encode_wide_batch_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ DqDevTable TV,
                             const __grid_constant__ DqPairEnc PK, const __grid_constant__ DqPairEnc PV, const DqEncodeArgs a) {
     extern __shared__ __align__(16) uint8_t dyn[];
-    __shared__ EncTable T;
+    __shared__ __align__(16) EncTable T;
     __shared__ __align__(16) WideShared W;
     __shared__ uint32_t s_hdr[kWB], s_flags[kWB], s_xs[kWB], s_k[kWB];
     dqdev::pdl_launch_dependents();
@@ -1257,8 +814,11 @@ cudaError_t dq_launch_means(const DqDevTable& tk, const void* k_bf16, int T, int
 static long long batch_min_streams(long long dflt) { return dq_opt_encode_batch_min(dflt); }
 
 cudaError_t dq_launch_encode(const DqDevTable& tk, const DqDevTable& tv, const DqPairEnc& pk, const DqPairEnc& pv,
-                             const DqEncodeArgs& a, cudaStream_t st) {
+                             const DqEncodeArgs& args, cudaStream_t st) {
+    DqEncodeArgs a = args;
     const long long warps = (long long)a.T * a.Hkv;
+    // umulhi(n, ceil(2^32 / d)) = n / d for every n < 2^32 / d
+    a.hkv_magic = (a.Hkv > 1 && warps < (1LL << 32) / a.Hkv) ? (uint32_t)(((1ull << 32) + a.Hkv - 1) / a.Hkv) : 0u;
     if (warps == 0 || (!a.do_k && !a.do_v)) return cudaSuccess;
     if (tk.hs > 1) {   // token-wide streams: CTAs of hs warps; few streams: one per CTA, many: 32 per CTA
         const long long streams = warps / tk.hs;
@@ -1277,9 +837,8 @@ cudaError_t dq_launch_encode(const DqDevTable& tk, const DqDevTable& tv, const D
     const unsigned blocks = (unsigned)((warps + kEncWarps - 1) / kEncWarps);
     const bool pair = tk.pair != 0;   // the caller has checked that both tables agree
     const dim3 kinds(1, (a.do_k && a.do_v) ? 2 : 1);
-    if (!a.step_flags && warps >= batch_min_streams(4LL * 148 * kB32 * 4))   // enough streams to fill the GPU several times
-        return dq_launch_pdl(pair ? dq_encode_batch32_kernel<kB32PairMinBlocks, true> : dq_encode_batch32_kernel<DQ_B32_MINB, false>,
-                             dim3((unsigned)((warps + kB32 - 1) / kB32), kinds.y), dim3(kB32Warps * 32), 0, st, tk, tv, pk, pv, a);
+    if (!a.step_flags && warps >= batch_min_streams(4LL * 148 * kDqEncodeBatchStreams * 4))   // enough streams to fill the GPU several times
+        return dq_launch_encode_batch(tk, tv, pk, pv, a, st);
     if (a.step_flags) {   // decode step: big CTAs, so that few SMs are kept from the attention kernel
         constexpr int kStepWarps = DQ_STEP_ENC_WARPS;
         return dq_launch_pdl(pair ? dq_encode_kernel<1, kStepWarps, true> : dq_encode_kernel<1, kStepWarps, false>,

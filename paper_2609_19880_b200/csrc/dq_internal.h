@@ -17,6 +17,15 @@ struct DqDevTable {
     uint32_t enc_aux[DQ_MAX_LEVELS];  // bias | (256 - f) << 10 | rsh << 19, bias = c (+ 255 when f = 1)
     float r[DQ_MAX_LEVELS];      // ideal cost in bits     (Algorithm 1)
     uint32_t R[DQ_MAX_LEVELS];   // ceil(r * 65536)
+    // Encoder, thresholds of Drift (dq_drift.cuh): edge e of a side (0: below the central level, 1: above) is the step
+    // from its level mstar -+ (e + 1) to the next inner one.
+    float edge_inv[2][DQ_MAX_LEVELS / 2];    // 1 / (r_outer - r_inner); 1e20 for a central pair of equal costs; 0 where there is no such edge
+    float edge_off[2][DQ_MAX_LEVELS / 2];    // -(e + 1/2) edge_inv; -1 where there is no such edge
+    uint32_t edge_dR[2][DQ_MAX_LEVELS / 2];  // R_outer - R_inner
+    float edge_xm[2], edge_inv_m[2];         // outermost two edges merge from this position on; their common 1 / (sum of differences)
+    float edge_inv_max, edge_rho;            // largest of the other inverses; max r times it
+    uint32_t edge_few;                       // 2.5 x the largest R difference
+    int drift_fast;                          // thresholds usable: 0 no, 1 yes, 2 yes with the merged outermost pair
     uint32_t lut[256];           // f << 24 | fp16(level) << 8 | (z - c)   (Algorithm 2)
                                  // pair: code(b) << 24 | f << 16 | code(a) << 8 | (z - c), code = high byte of fp16(level)
 };
@@ -59,6 +68,7 @@ struct DqEncodeArgs {
     float* mean_scale;
     uint32_t* status;
     int T, Hkv, max_windows, mean_mode, do_k, do_v;
+    uint32_t hkv_magic;      // ceil(2^32 / Hkv): stream / Hkv by a high multiply; 0: not exact for this call's streams
     const float* rope_cos;   // [positions][64], nullable: keys are handed over before their rotary embedding
     const float* rope_sin;
     int rope_style;          // 0 none, DQ_ROPE_HALF, DQ_ROPE_PAIRS

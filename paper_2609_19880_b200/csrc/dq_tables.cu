@@ -161,6 +161,47 @@ double table_entropy(const dq_table_info& t) {
     return h;
 }
 
+// Thresholds of Drift (dq_drift.cuh).  They replace the sweeps where the steps from an outer level to the next inner
+// one happen in order as lambda grows, whatever the value: the cost differences of a side must not fall
+// outwards, except that the outermost one may (its step then merges with the next one from some
+// position on), and no two levels of a side may cost the same, except the two central ones.
+void drift_edges(const dq_table_info& t, DqDevTable& d) {
+    const int centre = (t.levels - 1) / 2;
+    bool ok = t.mstar == centre, merge = false;
+    float rmax = 0.f;
+    uint32_t dR_max = 0;
+    d.edge_inv_max = 0.f;
+    for (int m = 0; m < t.levels; ++m) rmax = std::max(rmax, t.r[m]);
+    for (int side = 0; side < 2; ++side) {
+        const int ne = side ? t.levels - 1 - centre : centre, step = side ? 1 : -1;
+        double dr[DQ_MAX_LEVELS];
+        d.edge_xm[side] = INFINITY;
+        for (int e = 0; e < DQ_MAX_LEVELS / 2; ++e) { d.edge_inv[side][e] = 0.f; d.edge_off[side][e] = -1.f; d.edge_dR[side][e] = 0u; }
+        for (int e = 0; e < ne; ++e) {
+            const int in = centre + step * e, outl = in + step;
+            dr[e] = (double)t.r[outl] - (double)t.r[in];
+            d.edge_dR[side][e] = t.R[outl] - t.R[in];
+            const bool central_pair = side == 1 && e == 0 && t.levels % 2 == 0;
+            // equal costs: the central pair's step never happens; elsewhere (not ok) only the sign of y counts
+            const double inv = dr[e] > 0.0 ? 1.0 / dr[e] : dr[e] == 0.0 && central_pair ? 1e20 : 1.0;
+            d.edge_inv[side][e] = (float)inv;
+            d.edge_off[side][e] = (float)(-(e + 0.5) * inv);
+            if (dr[e] < 0.0 || (dr[e] == 0.0 && !central_pair)) ok = false;
+            if (inv < 1e20) d.edge_inv_max = std::max(d.edge_inv_max, (float)inv);
+            if (dr[e] > 0.0) dR_max = std::max(dR_max, d.edge_dR[side][e]);
+            if (e > 0 && dr[e] < dr[e - 1]) {
+                if (e != ne - 1 || (e > 1 && 0.5 * (dr[e] + dr[e - 1]) < dr[e - 2])) ok = false;
+                d.edge_xm[side] = (float)(dr[e] / (dr[e - 1] - dr[e]));
+                d.edge_inv_m[side] = (float)(1.0 / (dr[e] + dr[e - 1]));
+                merge = true;
+            }
+        }
+    }
+    d.edge_rho = rmax * d.edge_inv_max;
+    d.edge_few = dR_max * 5 / 2;
+    d.drift_fast = ok ? (merge ? 2 : 1) : 0;
+}
+
 }  // namespace
 
 int dq_host_build(int levels, double bits_per_elem, const dq_table_opts* opts, dq_tables* out) {
@@ -248,6 +289,7 @@ int dq_host_build(int levels, double bits_per_elem, const dq_table_opts* opts, d
         d.r[m] = t.r[m];
         d.R[m] = t.R[m];
     }
+    drift_edges(t, d);
     if (pair) {
         uint32_t c = 0;
         for (int u = 0; u < levels * levels; ++u) {
