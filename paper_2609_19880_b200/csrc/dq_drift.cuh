@@ -9,7 +9,7 @@
 //     lambda = 2 s^2 y,   y = x / (r_outer - r_inner),   x = distance from the edge's midpoint in level units.
 // So the code length at lambda is the all-central length plus the R differences of the edges with
 // 2 s^2 y > lambda, and J is the cell of the largest y at which the sum over the edges not below it exceeds what
-// the budget leaves: an order statistic, found by interpolation on y (about four sums and two maxima).
+// the budget leaves: an order statistic, found by interpolation on y (about four sums over 4 values per lane, then one or two maxima).
 //
 // The records are defined by the binary32 costs fma(lambda, r_m, D_m), lowest index among equal ones, at the
 // rounded lambdas.  Rounding moves a step by E level units in x and by a relative wA (both bounded below).  The
@@ -31,7 +31,7 @@ using dqdev::kFullMask;
 struct EncTable {
     float r[DQ_MAX_LEVELS];
     uint32_t R[DQ_MAX_LEVELS];
-    // Eq. rans Enc: {rcp, thr, bias, (2^p - f) | rsh << 16}: floor(x / f) = umulhi(x, rcp) >> rsh, bias = c (+ 255 when
+    // Eq. rans Enc: {rcp, thr, bias, (2^p - f) << 5 | rsh}: floor(x / f) = umulhi(x, rcp) >> rsh, bias = c (+ 255 when
     // f = 1), thr = f << (sigma - 9) = f L: renormalise while the state is not below it
     uint4 enc[DQ_MAX_PAIRS];
     uint2 prk[DQ_MAX_PAIRS];       // pairs: {bits of r_u, ceil(65536 r_u) << 8 | u}
@@ -79,6 +79,11 @@ __device__ __forceinline__ float lg2_approx(float x) {
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 __device__ __forceinline__ float exp2_approx(float x) {
@@ -164,32 +169,23 @@ __device__ __forceinline__ bool drift_thresholds(const EncTable& T, const Group&
         dmin = __uint_as_float(grp.min(__float_as_uint(dmin)));
         const float Dn = fmaf(reach, reach, -dmin * dmin);               // (max D - min D) / s^2
 
-        // Bracket [ya, yb]: the sum over y > ya exceeds cap, the one over y > yb does not.  Interpolated (leaning
-        // towards ya, the sums being convex; an end that stays is weighted down) until few edges are between.
-        float ya = 0.f, yb = (fmaxf(vmax - (float)kC, (float)kC - vmin) - 0.49f) * T.inv_max, fb = (float)cap, fa = (float)(Wa - cap);
+        // Bracket [ya, yb]: the sum over y > ya exceeds cap, the one over y > yb does not.  Interpolated, leaning towards
+        // ya (the sums are convex), until few edges are between: 4.3 sums on average, halving takes 7.
+        float ya = 0.f, yb = (fmaxf(vmax - (float)kC, (float)kC - vmin) - 0.49f) * T.inv_max;
         uint32_t Wb = 0;
-        {
-            int last = 0;
 #pragma unroll 1
-            for (int it = 0; it < 16 && Wa - Wb > T.dR_few; ++it) {
-                const float t = fminf(fmaxf(0.85f * fa * rcp_approx(fa + fb), 0.02f), 0.98f);
-                const float ym = fmaf(yb - ya, t, ya);
-                w = 0;
+        for (int it = 0; it < 14 && Wa - Wb > T.dR_few; ++it) {
+            const float t = 0.85f * (float)(int)(Wa - cap) * rcp_approx((float)(int)(Wa - Wb));
+            const float ym = fmaf(yb - ya, fminf(fmaxf(t, 0.05f), 0.95f), ya);
+            w = 0;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int e = 0; e < kHigh; ++e) add_if_greater(w, y[i][e], ym, dR[i][e]);
-                w = grp.add(w);
-                if (w > cap) {
-                    ya = ym; Wa = w; fa = (float)(w - cap);
-                    if (last == 1) fb *= 0.5f;
-                    last = 1;
-                } else {
-                    yb = ym; Wb = w; fb = (float)(cap - w);
-                    if (last == 2) fa *= 0.5f;
-                    last = 2;
-                }
-            }
+                for (int e = 0; e < kHigh; ++e) add_if_greater(w, y[i][e], ym, dR[i][e]);
+            w = grp.add(w);
+            const bool over = w > cap;
+            ya = over ? ym : ya; Wa = over ? w : Wa;
+            yb = over ? yb : ym; Wb = over ? Wb : w;
         }
         // then down from yb, one edge at a time
         float yc = __uint_as_float(__float_as_uint(yb) + 1u);
@@ -201,7 +197,7 @@ __device__ __forceinline__ bool drift_thresholds(const EncTable& T, const Group&
 #pragma unroll
                 for (int e = 0; e < kHigh; ++e) max_if_less(m, y[i][e], yc);
             yc = __uint_as_float(grp.max(__float_as_uint(m)));
-            if (it == 24 || !(yc > 0.f)) return false;
+            if (it == 40 || !(yc > 0.f)) return false;
             w = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -209,28 +205,43 @@ __device__ __forceinline__ bool drift_thresholds(const EncTable& T, const Group&
                 for (int e = 0; e < kHigh; ++e) add_if_not_less(w, y[i][e], yc, dR[i][e]);
             if (grp.add(w) > cap) break;
         }
-        // yc again, from the rounded level positions that the costs use: E becomes 3 units of 2^-24 (not when merged)
-        float yr = 0.f;
+        // yc again, from the rounded level positions that the costs use: E becomes 3 units of 2^-24.  Only for a single,
+        // unmerged edge; it leaves y[][] here, being taken at lambda_{J+1} by construction.
+        float zc = 0.f, code = 0.f;   // its value, and (edge + 1) with the sign of its side
+        uint32_t equal = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int e = 0; e < kHigh; ++e)
-                if (y[i][e] == yc) {
-                    const int up = a[i] >= 0.f ? 1 : 0;
-                    const float in = up ? (float)(kC + e) : (float)(kC - e), dir = up ? 1.f : -1.f;
-                    const float di = z[i] - fmaf(in, s, o), dq = z[i] - fmaf(in + dir, s, o);
-                    yr = ((di - dq) * inv) * ((di + dq) * inv) * 0.5f * __uint_as_float(T.edge[up][e].x);
-                }
-        yr = __uint_as_float(grp.max(__float_as_uint(fmaxf(yr, 0.f))));
-        const bool refined = T.fast == 1 && yr > 0.f;
+            for (int e = 0; e < kHigh; ++e) {
+                const bool is = y[i][e] == yc;
+                zc = is ? z[i] : zc;
+                code = is ? copysignf((float)(e + 1), a[i]) : code;
+                y[i][e] = is ? 0.f : y[i][e];
+                equal += is ? 1u : 0u;
+            }
+        float yr = 0.f;
+        if (equal) {
+            const float dir = copysignf(1.f, code), outer = (float)kC + code;
+            const float di = zc - fmaf(outer - dir, s, o), dq = zc - fmaf(outer, s, o);
+            yr = fmaxf(((di - dq) * inv) * ((di + dq) * inv) * 0.5f * __uint_as_float(T.edge[dir > 0.f ? 1 : 0][(int)fabsf(code) - 1].x), 0.f);
+        }
+        yr = __uint_as_float(grp.max(__float_as_uint(yr)));
+        const bool refined = grp.add(equal) == 1u && T.fast == 1 && yr > 0.f;
         // cell of yc (grid units from 3072 on: less to round), lambda_{J+1} / (2 s^2)
         const float wA = 4e-4f + 1.5f * 148.f * 0x1p-24f * (2.f * mag + 4.f * reach + 2.f * T.rho);
-        const float lgD = log2f(Dn) - 8.f;
+        const float lgD = log2f(Dn) - 8.f, ryc = rcp_approx(yc);
         const float u = kG * (lg2_approx(refined ? yr : yc) - lgD);
-        const float wc = fmaf(148.f * T.inv_max * (refined ? 4.5f * 0x1p-24f : E), rcp_approx(yc), wA);
+        const float wc = fmaf(148.f * T.inv_max * (refined ? 4.5f * 0x1p-24f : E), ryc, wA);
         const float J = floorf(u - wc);
         tie = floorf(u + wc) != J || J < -3070.f || J > 1020.f;
         yf = exp2_approx(fmaf(J + 1.f, 1.f / kG, lgD));
+        if (refined && u - fmaf(148.f * band, 2.f * ryc, wA) < J) {   // the unrefined edges next to yc may be below lambda_J
+            const float yJ = exp2_approx(fmaf(J, 1.f / kG, lgD)), bJ = fmaf(yJ, wA * (1.f / 148.f), band);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int e = 0; e < kHigh; ++e) tie |= fabsf(y[i][e] - yJ) <= bJ;
+        }
         band = fmaf(yf, wA * (1.f / 148.f), band);
     }
     uint32_t lev[4];

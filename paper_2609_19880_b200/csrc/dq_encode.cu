@@ -218,7 +218,7 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
             ++k;
             xs >>= 8;
         }
-        xs = (__umulhi(xs, en.x) >> (en.w >> 16)) * (en.w & 0xffffu) + (xs + en.z);
+        xs = __funnelshift_r(__umulhi(xs, en.x), 0u, en.w) * (en.w >> 5) + (xs + en.z);
     }
     __syncwarp();
     asm volatile("" ::: "memory");

@@ -70,7 +70,7 @@ __device__ __forceinline__ void load_enc_table(EncTable& T, const DqDevTable& TK
             aux = is_v ? TV.enc_aux[i] : TK.enc_aux[i];
         }
         const uint32_t cmpl = (aux >> 10) & 511u;
-        T.enc[i] = make_uint4(rcp, (256u - cmpl) << (sigma - 9), aux & 1023u, cmpl | ((aux >> 19) << 16));
+        T.enc[i] = make_uint4(rcp, (256u - cmpl) << (sigma - 9), aux & 1023u, cmpl << 5 | aux >> 19);
     }
     if (i == 0) {
         T.M = is_v ? TV.M : TK.M; T.rec = is_v ? TV.rec : TK.rec; T.mstar = is_v ? TV.mstar : TK.mstar;
@@ -250,6 +250,15 @@ __device__ __forceinline__ uint32_t drift_pair(const EncTable& T, const float (&
 __device__ __forceinline__ int tok_pos(const DqEncodeArgs& a, int t) { return a.step_seq_lens ? a.step_seq_lens[t] - 1 : a.pos[t]; }
 __device__ __forceinline__ int tok_seq(const DqEncodeArgs& a, int t) { return a.step_seq_lens ? t : a.seq_id[t]; }
 
+// One step of Eq. rans Enc with the entry `en` of EncTable::enc: a byte of the state goes to shared memory at `dst`,
+// which advances by `stride`, when the state is not below en.y (at most once: x < 2^8 L <= 2^8 (f L)).
+template <int STRIDE>
+__device__ __forceinline__ void rans_step(uint32_t& x, uint32_t& dst, const uint4 en) {
+    asm volatile("{.reg .pred p; setp.ge.u32 p, %0, %2; @p st.shared.u8 [%1], %0; @p add.u32 %1, %1, %3; @p shr.u32 %0, %0, 8;}"
+                 : "+r"(x), "+r"(dst) : "r"(en.y), "n"(STRIDE) : "memory");
+    x = __funnelshift_r(__umulhi(x, en.x), 0u, en.w) * (en.w >> 5) + (x + en.z);   // the shift uses en.w mod 32
+}
+
 struct StreamQuantised {
     uint32_t hdr0;      // s fp16 | o fp16 << 16
     uint32_t flags;     // 1: all-central fallback, 2: constant stream, 4: refit rejected
@@ -324,12 +333,12 @@ __device__ __forceinline__ bool refit_integers(const float (&z)[4], float zabs, 
     const int SA = (int)(__reduce_add_sync(kFull, a) - kN * kMagic);
     const int SB = (int)(__reduce_add_sync(kFull, b) - (uint32_t)Sm * kMagic);
     if (den <= 0) return false;
-    const long long num = (long long)kN * SB - (long long)Sm * SA;
-    const float sd = (float)num * __frcp_rn((float)den);                              // in units
+    const float nb = (float)kN * (float)SB, ma = (float)Sm * (float)SA, rd = dqdrift::rcp_approx((float)den);
+    const float sd = (nb - ma) * rd;                                                  // in units
     const float t = sd * (float)Sm;
     const float od = ((float)SA - t) * (1.f / kN);
     // |sum of (n m - Sm) errors| <= n sqrt(den) / 2; binary32 roundings
-    const float es = 0.51f * kN * rsqrtf((float)den) + 0x1p-21f * fabsf(sd);
+    const float es = 0.52f * kN * dqdrift::sqrt_approx(rd) + 0x1p-22f * rd * (fabsf(nb) + fabsf(ma)) + 0x1p-21f * fabsf(sd);
     const float eo = 0.51f + (es * (float)Sm + 0x1p-22f * (fabsf((float)SA) + fabsf(t))) * (1.f / kN);
     const __half2 lo = __floats2half2_rn((sd - es) * unit, (od - eo) * unit), hi = __floats2half2_rn((sd + es) * unit, (od + eo) * unit);
     hdr = *reinterpret_cast<const uint32_t*>(&lo);

@@ -110,21 +110,19 @@ dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_con
     }
     __syncthreads();
     if (wib == 0 && lane < ns) {   // rANS, Eq. (rans) Enc on the symbols from the last one back; lane = stream
-        uint32_t xs = 1u << (T.sigma - 9), k = 0;
+        uint32_t xs = 1u << (T.sigma - 9);
+        const uint32_t dst0 = dqdev::smem_addr(s_bytesT) + lane;
+        uint32_t dst = dst0;   // at most one byte per symbol: 128 rows of kB32 bytes suffice
 #pragma unroll 1
         for (int jw = (PAIR ? kN / 2 : kN) / 4 - 1; jw >= 0; --jw) {
             const uint32_t m4 = s_sym[lane * kB32SymWords + jw];
+            uint4 en[4];
 #pragma unroll
-            for (int b = 3; b >= 0; --b) {
-                const uint4 en = T.enc[(m4 >> (8 * b)) & 0xffu];
-                if (xs >= en.y) {   // at most once: xs < 2^8 L <= 2^8 * (f L)
-                    if (k < DQ_MAX_REC_BYTES) s_bytesT[k * kB32 + lane] = (uint8_t)xs;   // the budget test keeps k < rec - 8
-                    ++k;
-                    xs >>= 8;
-                }
-                xs = (__umulhi(xs, en.x) >> (en.w >> 16)) * (en.w & 0xffffu) + (xs + en.z);
-            }
+            for (int b = 0; b < 4; ++b) en[b] = T.enc[(m4 >> (8 * b)) & 0xffu];
+#pragma unroll
+            for (int b = 3; b >= 0; --b) rans_step<kB32>(xs, dst, en[b]);
         }
+        const uint32_t k = (dst - dst0) / kB32;
         s_xs[lane] = xs;
         s_k[lane] = k;
         if (a.status) atomicMax(a.status + 3, 4u + (uint32_t)(T.sigma >> 3) + k);
@@ -134,11 +132,10 @@ dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_con
     const uint32_t rec_magic = 0xffffffffu / (uint32_t)rec + 1u;   // idx / rec by a high multiply: idx < 2^13
     for (int idx = threadIdx.x; idx < ns * rec; idx += blockDim.x) {   // records out: header, state, k bytes, then zeros
         const int si = (int)__umulhi((uint32_t)idx, rec_magic), i = idx - si * rec;
-        const int k = (int)s_k[si], used = min(pay + k, rec);
-        uint8_t v = 0;
-        if (i < 4) v = (uint8_t)(s_hdr[si] >> (8 * i));
-        else if (i < pay) v = (uint8_t)(s_xs[si] >> (8 * (i - 4)));
-        else if (i < used) v = s_bytesT[(k - 1 - (i - pay)) * kB32 + si];   // emitted last = read first
+        const int k = (int)s_k[si], at = k - 1 - (i - pay);   // emitted last = read first
+        const uint32_t tail = s_bytesT[min(max(at, 0), kN) * kB32 + si];
+        const uint32_t head = i < 4 ? s_hdr[si] >> (8 * i) : s_xs[si] >> (8 * (i & 3));
+        const uint8_t v = (uint8_t)(i < pay ? head : at >= 0 ? tail : 0u);
         reinterpret_cast<uint8_t*>(s_rec[si])[i] = v;
     }
     if (second) dqdev::pdl_wait_prior_grid();   // the first kind's kernel: whoever waits for this one may read both
