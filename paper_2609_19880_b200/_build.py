@@ -23,6 +23,7 @@ _SOURCES = [
     ("dq_microbench.cu", []),
     ("dq_encode.cu", ["-fmad=false"]),
     ("dq_encode_batch.cu", ["-fmad=false"]),
+    ("dq_encode_wide.cu", ["-fmad=false"]),
 ]
 _COMMON = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
            "-Xcompiler", "-fPIC", "-I", _INC, "-I", _CSRC]

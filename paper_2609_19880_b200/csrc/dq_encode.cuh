@@ -49,17 +49,17 @@ __device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, const floa
 
 // ------------------------------------------------------------------------ drift
 
-// Table of one tensor kind into shared memory (threads 0 .. DQ_MAX_PAIRS - 1 and thread 0).
+// Table of one tensor kind into shared memory, by all threads of the CTA (at least 32).
 __device__ __forceinline__ void load_enc_table(EncTable& T, const DqDevTable& TK, const DqDevTable& TV,
                                                const DqPairEnc& PK, const DqPairEnc& PV, bool is_v) {
     const int pair = is_v ? TV.pair : TK.pair, sigma = is_v ? TV.sigma : TK.sigma;
-    const int i = threadIdx.x;
     dqdrift::load_edges(T, TK, TV, is_v);
-    if (i < DQ_MAX_LEVELS) {
+    if (threadIdx.x < DQ_MAX_LEVELS) {
+        const int i = threadIdx.x;
         T.r[i] = is_v ? TV.r[i] : TK.r[i];
         T.R[i] = is_v ? TV.R[i] : TK.R[i];
     }
-    if (i < (pair ? DQ_MAX_PAIRS : DQ_MAX_LEVELS)) {
+    for (int i = threadIdx.x; i < (pair ? DQ_MAX_PAIRS : DQ_MAX_LEVELS); i += blockDim.x) {
         uint32_t rcp, aux;
         if (pair) {
             rcp = is_v ? PV.enc_rcp[i] : PK.enc_rcp[i];
@@ -72,7 +72,7 @@ __device__ __forceinline__ void load_enc_table(EncTable& T, const DqDevTable& TK
         const uint32_t cmpl = (aux >> 10) & 511u;
         T.enc[i] = make_uint4(rcp, (256u - cmpl) << (sigma - 9), aux & 1023u, cmpl << 5 | aux >> 19);
     }
-    if (i == 0) {
+    if (threadIdx.x == 0) {
         T.M = is_v ? TV.M : TK.M; T.rec = is_v ? TV.rec : TK.rec; T.mstar = is_v ? TV.mstar : TK.mstar;
         T.budget_bits = is_v ? TV.budget_bits : TK.budget_bits;
         T.has_mean = is_v ? TV.has_mean : TK.has_mean; T.rotate = is_v ? TV.rotate : TK.rotate;
@@ -310,45 +310,64 @@ __device__ __forceinline__ void carry_mean(const DqEncodeArgs& a, size_t mi, int
     if (lane == 0) a.mean_scale[mi] = sc;
 }
 
-// Least squares of z on the symbols from integer sums: the values are rounded to multiples of `unit` (2^-20 of the
-// power of two above the largest), so that every sum is one integer reduction.  The binary64 sums that
-// define the result differ from these by less than the two errors computed below; when both ends of the error
+// Least squares of z on the symbols from integer sums: the values are rounded to multiples of `unit` (2^-19 of the
+// power of two below the largest), so that every sum is one integer reduction.  The binary64 sums that
+// define the result differ from these by less than the two errors of refit_finish; when both ends of the error
 // interval round to the same fp16 pair, that is the pair (all but about one stream in 200).
-__device__ __forceinline__ bool refit_integers(const float (&z)[4], float zabs, uint32_t sym, uint32_t& hdr) {
-    constexpr uint32_t kMagic = 0x4b400000u;   // 1.5 2^23: the low bits of z / unit + 1.5 2^23 are the integer
-    if (!(zabs > 0x1p-60f && zabs < 0x1p60f)) return false;
+struct RefitScale {
+    float scale, unit;   // 1 / unit, unit
+    bool ok;
+};
+__device__ __forceinline__ RefitScale refit_scale(float zabs) {
     const uint32_t ex = __float_as_uint(zabs) & 0x7f800000u;                          // 2^e <= zabs < 2^(e + 1)
-    const float scale = __uint_as_float((254u << 23) - ex + (19u << 23));             // 2^(19 - e)
-    const float unit = __uint_as_float(ex - (19u << 23));                             // 2^(e - 19)
+    RefitScale r;
+    r.ok = zabs > 0x1p-60f && zabs < 0x1p60f;
+    r.scale = __uint_as_float((254u << 23) - ex + (19u << 23));                       // 2^(19 - e)
+    r.unit = __uint_as_float(ex - (19u << 23));
+    return r;
+}
+
+struct RefitSums {
+    int Sm, Smm, SA, SB;   // sums of m, m^2, z / unit, m z / unit over a warp's 128 values
+};
+__device__ __forceinline__ RefitSums refit_sums(const float (&z)[4], const RefitScale& sc, uint32_t sym) {
+    constexpr uint32_t kMagic = 0x4b400000u;   // 1.5 2^23: the low bits of z / unit + 1.5 2^23 are the integer
     uint32_t a = 0, b = 0;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const uint32_t zi = __float_as_uint(__fmaf_rn(z[e], scale, 12582912.f));
+        const uint32_t zi = __float_as_uint(__fmaf_rn(z[e], sc.scale, 12582912.f));
         a += zi;
         b += zi * ((sym >> (8 * e)) & 0xffu);
     }
     // sums of the levels and of their squares: < 2^11 and < 2^15
     const uint32_t both = __reduce_add_sync(kFull, __dp4a(sym, 0x01010101u, 0u) << 16 | __dp4a(sym, sym, 0u));
-    const int Sm = (int)(both >> 16), den = kN * (int)(both & 0xffffu) - Sm * Sm;
-    const int SA = (int)(__reduce_add_sync(kFull, a) - kN * kMagic);
-    const int SB = (int)(__reduce_add_sync(kFull, b) - (uint32_t)Sm * kMagic);
-    if (den <= 0) return false;
-    const float nb = (float)kN * (float)SB, ma = (float)Sm * (float)SA, rd = dqdrift::rcp_approx((float)den);
+    RefitSums r;
+    r.Sm = (int)(both >> 16);
+    r.Smm = (int)(both & 0xffffu);
+    r.SA = (int)(__reduce_add_sync(kFull, a) - kN * kMagic);
+    r.SB = (int)(__reduce_add_sync(kFull, b) - (uint32_t)r.Sm * kMagic);
+    return r;
+}
+
+// fp16 pair of the solution for n values, or false when its rounding is within the error of a tie.
+__device__ __forceinline__ bool refit_finish(const RefitScale& sc, float n, float SA, float SB, float Sm, float den, uint32_t& hdr) {
+    if (!(den > 0.f)) return false;
+    const float nb = n * SB, ma = Sm * SA, rd = dqdrift::rcp_approx(den), rn = 1.f / n;   // n is a constant or a small integer
     const float sd = (nb - ma) * rd;                                                  // in units
-    const float t = sd * (float)Sm;
-    const float od = ((float)SA - t) * (1.f / kN);
-    // |sum of (n m - Sm) errors| <= n sqrt(den) / 2; binary32 roundings
-    const float es = 0.52f * kN * dqdrift::sqrt_approx(rd) + 0x1p-22f * rd * (fabsf(nb) + fabsf(ma)) + 0x1p-21f * fabsf(sd);
-    const float eo = 0.51f + (es * (float)Sm + 0x1p-22f * (fabsf((float)SA) + fabsf(t))) * (1.f / kN);
-    const __half2 lo = __floats2half2_rn((sd - es) * unit, (od - eo) * unit), hi = __floats2half2_rn((sd + es) * unit, (od + eo) * unit);
+    const float t = sd * Sm;
+    const float od = (SA - t) * rn;
+    // |sum of (n m - Sm) errors| <= n sqrt(den) / 2, over den; binary32 roundings
+    const float es = 0.52f * n * dqdrift::sqrt_approx(rd) + 0x1p-22f * rd * (fabsf(nb) + fabsf(ma)) + 0x1p-21f * fabsf(sd);
+    const float eo = 0.51f + (es * Sm + 0x1p-21f * (fabsf(SA) + fabsf(t))) * rn;
+    const __half2 lo = __floats2half2_rn((sd - es) * sc.unit, (od - eo) * sc.unit), hi = __floats2half2_rn((sd + es) * sc.unit, (od + eo) * sc.unit);
     hdr = *reinterpret_cast<const uint32_t*>(&lo);
     return hdr == *reinterpret_cast<const uint32_t*>(&hi);
 }
 
-// The same from binary64 sums in a fixed order (lane order, then a butterfly), both parameters rounded once.
-static __device__ __noinline__ uint32_t refit_binary64(float z0, float z1, float z2, float z3, uint32_t sym, float s, float o) {
-    const float z[4] = {z0, z1, z2, z3};
-    double sa = (double)z[0], sb = __dmul_rn((double)(sym & 0xffu), (double)z[0]);
+// A warp's sums of z and m z in binary64, in the order that defines the result: a lane's values, then a butterfly.
+__device__ __forceinline__ void refit_sums_binary64(const float (&z)[4], uint32_t sym, double& sa, double& sb) {
+    sa = (double)z[0];
+    sb = __dmul_rn((double)(sym & 0xffu), (double)z[0]);
 #pragma unroll
     for (int e = 1; e < 4; ++e) {
         sa = __dadd_rn(sa, (double)z[e]);
@@ -359,6 +378,13 @@ static __device__ __noinline__ uint32_t refit_binary64(float z0, float z1, float
         sa = __dadd_rn(sa, __shfl_xor_sync(kFull, sa, d));
         sb = __dadd_rn(sb, __shfl_xor_sync(kFull, sb, d));
     }
+}
+
+// The refit from those sums, both parameters rounded once.
+static __device__ __noinline__ uint32_t refit_binary64(float z0, float z1, float z2, float z3, uint32_t sym, float s, float o) {
+    const float z[4] = {z0, z1, z2, z3};
+    double sa, sb;
+    refit_sums_binary64(z, sym, sa, sb);
     const int Sm = (int)__reduce_add_sync(kFull, __dp4a(sym, 0x01010101u, 0u)), Smm = (int)__reduce_add_sync(kFull, __dp4a(sym, sym, 0u));
     const int den = kN * Smm - Sm * Sm;
     double sd = (double)s, od = (double)o;
@@ -386,7 +412,10 @@ __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, co
     uint32_t sym = 0u;
     if (PAIR) drift_pair<M>(T, z, s, o, sym); else drift<M>(T, z, s, o, mn, mx, sym);
     uint32_t hdr;                                                   // Refit, fp16 metadata
-    if (!refit_integers(z, fmaxf(fabsf(mn), fabsf(mx)), sym, hdr)) hdr = refit_binary64(z[0], z[1], z[2], z[3], sym, s, o);
+    const RefitScale sc = refit_scale(fmaxf(fabsf(mn), fabsf(mx)));
+    const RefitSums h = refit_sums(z, sc, sym);
+    if (!sc.ok || !refit_finish(sc, (float)kN, (float)h.SA, (float)h.SB, (float)h.Sm, (float)(kN * h.Smm - h.Sm * h.Sm), hdr))
+        hdr = refit_binary64(z[0], z[1], z[2], z[3], sym, s, o);
     float sf = __half2float(__ushort_as_half((unsigned short)(hdr & 0xffffu))), of = __half2float(__ushort_as_half((unsigned short)(hdr >> 16)));
     if (!(isfinite(sf) && sf > 0.0f && isfinite(of))) {
         const __half s16 = __float2half_rn(s), o16 = __float2half_rn(o);
@@ -407,3 +436,6 @@ __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, co
 constexpr int kDqEncodeBatchStreams = 32;
 cudaError_t dq_launch_encode_batch(const DqDevTable& tk, const DqDevTable& tv, const DqPairEnc& pk, const DqPairEnc& pv,
                                    const DqEncodeArgs& a, cudaStream_t st);
+// Token-wide streams (dq_encode_wide.cu); per: streams per CTA, 0: by the size of the call.
+cudaError_t dq_launch_encode_wide(const DqDevTable& tk, const DqDevTable& tv, const DqPairEnc& pk, const DqPairEnc& pv,
+                                  const DqEncodeArgs& a, int per, cudaStream_t st);
