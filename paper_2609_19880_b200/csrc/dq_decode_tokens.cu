@@ -1,118 +1,249 @@
-// Check/debug decoder: Algorithm 2 on every record, one thread per stream, reading the
-// record straight from global memory.  Produces the symbols and the dequantised values
-// xhat = fma(m, s, o) (+ window mean for keys, Appendix A).  Not a performance path.
+// Export of records (dq_decode_tokens): Algorithm 2 with lane = stream out of shared memory, then the dequantised values
+// xhat = fma(m, s, o) (+ window mean for keys, Appendix A) and symbols written a head row per warp instruction.
+// Bound by the rANS chain's latency while a call has few streams (128 steps of about 90 cycles) and by the 640 bytes
+// written per stream when it has many; one thread per stream writing its own row ran at 5 % of the copy bandwidth.
 #include <cuda_fp16.h>
 
+#include "dq_device.cuh"
 #include "dq_internal.h"
 
 namespace {
 
-__global__ void __launch_bounds__(128)
-dq_decode_tokens_kernel(const __grid_constant__ DqDevTable T, const uint8_t* __restrict__ cont,
-                        const int8_t* __restrict__ mean_q, const float* __restrict__ mean_scale,
-                        int Wmax, const int32_t* __restrict__ seq_id, const int32_t* __restrict__ pos,
-                        const int32_t* __restrict__ slot, int n_tok, int Hkv,
-                        uint8_t* __restrict__ symbols, float* __restrict__ dequant) {
-    const long long sid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (sid >= (long long)n_tok * Hkv) return;
-    const int t = (int)(sid / Hkv), h = (int)(sid % Hkv);
-    const int sl = slot[t];
-    const uint8_t* rec = cont + (((size_t)(sl / DQ_PAGE_TOKENS) * Hkv + h) * DQ_PAGE_TOKENS +
-                                 (size_t)(sl % DQ_PAGE_TOKENS)) * T.rec;
-    const float s = __half2float(__ushort_as_half((unsigned short)(rec[0] | (rec[1] << 8))));
-    const float o = __half2float(__ushort_as_half((unsigned short)(rec[2] | (rec[3] << 8))));
-    // final state: sigma / 8 bytes, little-endian; the state interval starts at L = 2^(sigma - 9)
-    uint32_t x = (uint32_t)rec[4] | ((uint32_t)rec[5] << 8) | ((uint32_t)rec[6] << 16);
-    if (T.sigma == 32) x |= (uint32_t)rec[7] << 24;
-    int ptr = 4 + (T.sigma >> 3);
-    const uint32_t L = 1u << (T.sigma - 9);
-    const int8_t* mq = nullptr;
-    float msc = 0.f;
-    if (T.has_mean && mean_q) {
-        const size_t mi = ((size_t)seq_id[t] * Wmax + pos[t] / DQ_WINDOW_TOKENS) * Hkv + h;
-        mq = mean_q + mi * DQ_HEAD_DIM;
-        msc = mean_scale[mi];
-    }
-    auto emit = [&](int j, float lvl) {
-        if (symbols) symbols[sid * DQ_HEAD_DIM + j] = (uint8_t)(int)lvl;
-        if (dequant) {
-            float v = __fmaf_rn(lvl, s, o);
-            if (mq) v = __fadd_rn(v, __fmul_rn(msc, (float)mq[j]));
-            dequant[sid * DQ_HEAD_DIM + j] = v;
-        }
-    };
-    if (T.pair) {   // one step per pair of values: entry = code(b) << 24 | f << 16 | code(a) << 8 | (z - c)
-        for (int j = 0; j < DQ_HEAD_DIM; j += 2) {
-            const uint32_t e = T.lut[x & 255u];
-            x = ((e >> 16) & 255u) * (x >> 8) + (e & 255u);
-            if (x < L && ptr < T.rec) x = (x << 8) | rec[ptr++];  // at most one byte
-            emit(j, __half2float(__ushort_as_half((unsigned short)(e & 0xff00u))));
-            emit(j + 1, __half2float(__ushort_as_half((unsigned short)((e >> 16) & 0xff00u))));
-        }
-        return;
-    }
-    for (int j = 0; j < DQ_HEAD_DIM; ++j) {
-        const uint32_t e = T.lut[x & 255u];
-        x = (e >> 24) * (x >> 8) + (e & 255u);
-        if (x < L && ptr < T.rec) x = (x << 8) | rec[ptr++];  // at most one byte
-        emit(j, __half2float(__ushort_as_half((unsigned short)((e >> 8) & 0xffffu))));
+constexpr int kExportWarps = 4;
+constexpr int kSymRow = 33;   // words of a stream's symbol row: 128 bytes + pad
+
+struct ExportArgs {
+    const uint8_t* cont;
+    const int8_t* mean_q;
+    const float* mean_scale;
+    const int32_t* seq_id;
+    const int32_t* pos;
+    const int32_t* slot;
+    uint8_t* symbols;
+    float* dequant;
+    int Wmax, n_tok, Hkv;
+};
+
+constexpr int kLutCopies = 8;   // copies of the decode table, lane & 7 picks one: about two lanes per bank instead of 3.5
+
+// Decode table with integer symbols: f << 24 | symbol << 8 | (z - c); pairs: symbol = b << 4 | a.
+__device__ __forceinline__ void fill_lut(uint32_t* lut, const DqDevTable& T) {
+    auto level = [](uint32_t bits) { return (uint32_t)(int)__half2float(__ushort_as_half((unsigned short)bits)); };
+    for (int z = threadIdx.x; z < 256; z += blockDim.x) {
+        const uint32_t e = T.lut[z];
+        const uint32_t v = T.pair ? ((e << 8) & 0xff000000u) | level((e >> 16) & 0xff00u) << 12 | level(e & 0xff00u) << 8 | (e & 255u)
+                                  : (e & 0xff000000u) | level((e >> 8) & 0xffffu) << 8 | (e & 255u);
+#pragma unroll
+        for (int c = 0; c < kLutCopies; ++c) lut[z * kLutCopies + c] = v;
     }
 }
 
-// Token-wide streams: one thread per (token, group of hs heads), record read from the
-// word-interleaved page layout; symbols / dequantised values are written per head.
-__global__ void __launch_bounds__(128)
-dq_decode_tokens_wide_kernel(const __grid_constant__ DqDevTable T, const uint8_t* __restrict__ cont,
-                             const int8_t* __restrict__ mean_q, const float* __restrict__ mean_scale,
-                             int Wmax, const int32_t* __restrict__ seq_id, const int32_t* __restrict__ pos,
-                             const int32_t* __restrict__ slot, int n_tok, int Hkv,
-                             uint8_t* __restrict__ symbols, float* __restrict__ dequant) {
-    const int groups = Hkv / T.hs;
-    const long long sid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (sid >= (long long)n_tok * groups) return;
-    const int t = (int)(sid / groups), grp = (int)(sid % groups);
-    const int sl = slot[t];
-    const uint8_t* blk = cont + ((size_t)(sl / DQ_PAGE_TOKENS) * groups + grp) * ((size_t)T.rec_words * 64) +
-                         (size_t)(sl % DQ_PAGE_TOKENS) * 4;
-    auto byte_at = [&](int i) -> uint32_t { return blk[(size_t)(i >> 2) * 64 + (i & 3)]; };
-    const float s = __half2float(__ushort_as_half((unsigned short)(byte_at(0) | (byte_at(1) << 8))));
-    const float o = __half2float(__ushort_as_half((unsigned short)(byte_at(2) | (byte_at(3) << 8))));
-    uint32_t x = byte_at(4) | (byte_at(5) << 8) | (byte_at(6) << 16) | (byte_at(7) << 24);
+// Four rANS symbols packed into a word.  A symbol takes at most one byte: window(i) gives bytes i .. i + 3 of the record,
+// fetched before the serial chain needs them; a malformed record stops taking bytes at its end.
+template <typename Window>
+__device__ __forceinline__ uint32_t decode4(const uint32_t* lut, uint32_t& x, int& ptr, int rec, uint32_t L, Window window) {
+    uint32_t sym = 0, win = window(ptr);
+    const int left = rec - ptr;
+    int used = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t e = lut[(x & 255u) * kLutCopies];
+        x = (e >> 24) * (x >> 8) + (e & 255u);
+        const bool take = x < L && used < left;
+        x = take ? __byte_perm(x, win, 0x2104) : x;
+        win = take ? win >> 8 : win;
+        used += take ? 1 : 0;
+        sym |= ((e >> 8) & 255u) << (8 * i);
+    }
+    ptr += used;
+    return sym;
+}
+
+// The four levels of positions 4 lane .. 4 lane + 3 from a symbol row.
+template <bool PAIR>
+__device__ __forceinline__ uint32_t row_levels(const uint32_t* row, int lane) {
+    if (!PAIR) return row[lane];
+    const uint32_t two = reinterpret_cast<const uint16_t*>(row)[lane];   // pairs 2 lane, 2 lane + 1
+    const uint32_t lo = two & 0x0f0fu, hi = (two >> 4) & 0x0f0fu;        // levels of the even / odd values
+    return (lo & 255u) | (hi & 255u) << 8 | (lo >> 8) << 16 | (hi >> 8) << 24;
+}
+
+constexpr unsigned long long kNoMean = ~0ull;
+
+// Row of the mean arrays for (token t, head h), kNoMean without one.
+__device__ __forceinline__ unsigned long long mean_row(const DqDevTable& T, const ExportArgs& a, int t, int h) {
+    if (!T.has_mean || !a.mean_q) return kNoMean;
+    return ((unsigned long long)a.seq_id[t] * a.Wmax + a.pos[t] / DQ_WINDOW_TOKENS) * a.Hkv + h;
+}
+
+struct MeanPiece {
+    uint32_t q4;   // four INT8 means
+    float scale;
+};
+__device__ __forceinline__ MeanPiece load_mean(const ExportArgs& a, unsigned long long mi, int lane) {
+    MeanPiece m{0u, 0.f};
+    if (mi == kNoMean) return m;
+    m.scale = __ldg(a.mean_scale + mi);
+    const int8_t* p = a.mean_q + mi * DQ_HEAD_DIM + 4 * lane;
+    if ((reinterpret_cast<uintptr_t>(a.mean_q) & 3u) == 0) m.q4 = __ldg(reinterpret_cast<const uint32_t*>(p));
+    else
+        for (int e = 0; e < 4; ++e) m.q4 |= (uint32_t)(uint8_t)p[e] << (8 * e);
+    return m;
+}
+
+// Symbols and dequantised values of (token, head) row `at` / 128 by one warp.
+template <bool PAIR>
+__device__ __forceinline__ void write_row(const ExportArgs& a, const uint32_t* row, size_t at, bool has_mean, const MeanPiece& m, float s,
+                                          float o, int lane) {
+    const uint32_t m4 = row_levels<PAIR>(row, lane);
+    at += 4 * lane;
+    if (a.symbols) {
+        if ((reinterpret_cast<uintptr_t>(a.symbols) & 3u) == 0) *reinterpret_cast<uint32_t*>(a.symbols + at) = m4;
+        else
+            for (int e = 0; e < 4; ++e) a.symbols[at + e] = (uint8_t)(m4 >> (8 * e));
+    }
+    if (!a.dequant) return;
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        v[e] = __fmaf_rn((float)((m4 >> (8 * e)) & 255u), s, o);
+        if (has_mean) v[e] = __fadd_rn(v[e], __fmul_rn(m.scale, (float)(int)(int8_t)(m.q4 >> (8 * e))));
+    }
+    if ((reinterpret_cast<uintptr_t>(a.dequant) & 15u) == 0) *reinterpret_cast<float4*>(a.dequant + at) = make_float4(v[0], v[1], v[2], v[3]);
+    else
+        for (int e = 0; e < 4; ++e) a.dequant[at + e] = v[e];
+}
+
+// Per token-head streams: every warp takes 32 consecutive streams on its own.
+template <bool PAIR>
+__global__ void __launch_bounds__(kExportWarps * 32)
+dq_decode_tokens_kernel(const __grid_constant__ DqDevTable T, const ExportArgs a) {
+    extern __shared__ __align__(16) uint32_t dyn[];
+    __shared__ uint32_t lut_all[256 * kLutCopies];
+    fill_lut(lut_all, T);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t* lut = lut_all + (lane & (kLutCopies - 1));
+    const int rec = T.rec, row_words = ((rec + 10) >> 2) | 1;   // aligned words around a record and 4 bytes more; odd: lanes spread over the banks
+    uint32_t* recs = dyn + warp * 32 * (row_words + kSymRow);
+    uint32_t* syms = recs + 32 * row_words;
+    const long long total = (long long)a.n_tok * a.Hkv, first = ((long long)blockIdx.x * kExportWarps + warp) * 32;
+    const int ns = (int)min(32LL, total - first);
+    if (ns <= 0) return;
+    // lane = stream: where its record is
+    unsigned long long src = 0, mi = kNoMean;
+    if (lane < ns) {
+        int t, h;
+        t = (int)((first + lane) / a.Hkv);
+        h = (int)(first + lane - (long long)t * a.Hkv);
+        const int sl = a.slot[t];
+        src = (unsigned long long)(a.cont + (((size_t)(sl / DQ_PAGE_TOKENS) * a.Hkv + h) * DQ_PAGE_TOKENS + (size_t)(sl % DQ_PAGE_TOKENS)) * rec);
+        mi = mean_row(T, a, t, h);
+    }
+#pragma unroll 8
+    for (int i = 0; i < ns; ++i) {   // records into shared memory, a record's aligned words per warp instruction
+        const unsigned long long p = __shfl_sync(0xffffffffu, src, i);
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(p & ~3ull);
+        const int words = (int)((p & 3ull) + rec + 3) >> 2;
+        for (int k = lane; k < words; k += 32) recs[i * row_words + k] = __ldg(w + k);
+    }
+    __syncwarp();
+    float s = 0.f, o = 0.f;
+    if (lane < ns) {
+        const uint8_t* r = reinterpret_cast<const uint8_t*>(recs + lane * row_words) + (src & 3ull);
+        s = __half2float(__ushort_as_half((unsigned short)(r[0] | (r[1] << 8))));
+        o = __half2float(__ushort_as_half((unsigned short)(r[2] | (r[3] << 8))));
+        // final state: sigma / 8 bytes, little-endian; the state interval starts at L = 2^(sigma - 9)
+        uint32_t x = (uint32_t)r[4] | ((uint32_t)r[5] << 8) | ((uint32_t)r[6] << 16);
+        if (T.sigma == 32) x |= (uint32_t)r[7] << 24;
+        int ptr = 4 + (T.sigma >> 3);
+        const uint32_t L = 1u << (T.sigma - 9);
+        const uint32_t base = dqdev::smem_addr(r);
+        auto window = [&](int i) -> uint32_t { return dqdev::lds32_unaligned(base + i); };
+#pragma unroll 1
+        for (int j = 0; j < (PAIR ? 16 : 32); ++j) syms[lane * kSymRow + j] = decode4(lut, x, ptr, rec, L, window);
+    }
+    __syncwarp();
+    constexpr int kRows = 8;   // mean loads in flight
+    for (int i0 = 0; i0 < ns; i0 += kRows) {
+        MeanPiece m[kRows];
+        bool hm[kRows];
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            const unsigned long long mu = __shfl_sync(0xffffffffu, mi, min(i0 + u, ns - 1));
+            hm[u] = mu != kNoMean;
+            m[u] = load_mean(a, mu, lane);
+        }
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            const int i = i0 + u;
+            const float su = __shfl_sync(0xffffffffu, s, i & 31), ou = __shfl_sync(0xffffffffu, o, i & 31);
+            if (i < ns) write_row<PAIR>(a, syms + i * kSymRow, (size_t)(first + i) * DQ_HEAD_DIM, hm[u], m[u], su, ou, lane);
+        }
+    }
+}
+
+// Token-wide streams: a CTA takes 32 consecutive streams (token, group of hs heads).  Warp 0 decodes, lane =
+// stream, a head's 128 values at a time into one of two symbol tiles; the other warps write the head before.
+template <bool PAIR>
+__global__ void __launch_bounds__(kExportWarps * 32)
+dq_decode_tokens_wide_kernel(const __grid_constant__ DqDevTable T, const ExportArgs a) {
+    extern __shared__ __align__(16) uint32_t dyn[];
+    __shared__ uint32_t lut_all[256 * kLutCopies], tile[2][32 * kSymRow];
+    __shared__ int s_t[32], s_grp[32];
+    __shared__ float s_s[32], s_o[32];
+    __shared__ unsigned long long s_src[32], s_mi[32];
+    fill_lut(lut_all, T);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t* lut = lut_all + (lane & (kLutCopies - 1));
+    const int groups = a.Hkv / T.hs, rw = T.rec_words;
+    const long long total = (long long)a.n_tok * groups, first = (long long)blockIdx.x * 32;
+    const int ns = (int)min(32LL, total - first);
+    if (threadIdx.x < ns) {
+        const int t = (int)((first + lane) / groups), grp = (int)(first + lane - (long long)t * groups), sl = a.slot[t];
+        s_t[lane] = t;
+        s_grp[lane] = grp;
+        s_mi[lane] = mean_row(T, a, t, 0);
+        s_src[lane] = (unsigned long long)(a.cont + ((size_t)(sl / DQ_PAGE_TOKENS) * groups + grp) * ((size_t)rw * 64) + (size_t)(sl % DQ_PAGE_TOKENS) * 4);
+    }
+    __syncthreads();
+    const bool words_ok = (reinterpret_cast<uintptr_t>(a.cont) & 3u) == 0;
+    for (int i = threadIdx.x; i < rw * 32; i += blockDim.x) {   // [word][stream]: consecutive lanes, mostly adjacent slots
+        const int st = i & 31;
+        if (st >= ns) continue;
+        const uint8_t* p = reinterpret_cast<const uint8_t*>(s_src[st]) + (size_t)(i >> 5) * 64;
+        dyn[i] = words_ok ? __ldg(reinterpret_cast<const uint32_t*>(p))
+                          : (uint32_t)p[0] | (uint32_t)p[1] << 8 | (uint32_t)p[2] << 16 | (uint32_t)p[3] << 24;
+    }
+    __syncthreads();
+    auto byte = [&](int i) -> uint32_t { return (dyn[(i >> 2) * 32 + lane] >> (8 * (i & 3))) & 255u; };
+    auto window = [&](int i) -> uint32_t {
+        const int w0 = i >> 2;
+        return __funnelshift_r(dyn[min(w0, rw - 1) * 32 + lane], dyn[min(w0 + 1, rw - 1) * 32 + lane], 8 * (i & 3));
+    };
+    uint32_t x = 1u << 23;
     int ptr = 8;
-    for (int k = 0; k < T.hs; ++k) {
-        const int h = grp * T.hs + k;
-        const int8_t* mq = nullptr;
-        float msc = 0.f;
-        if (T.has_mean && mean_q) {
-            const size_t mi = ((size_t)seq_id[t] * Wmax + pos[t] / DQ_WINDOW_TOKENS) * Hkv + h;
-            mq = mean_q + mi * DQ_HEAD_DIM;
-            msc = mean_scale[mi];
-        }
-        const size_t dst = ((size_t)t * Hkv + h) * DQ_HEAD_DIM;
-        auto emit = [&](int j, float lvl) {
-            if (symbols) symbols[dst + j] = (uint8_t)(int)lvl;
-            if (dequant) {
-                float v = __fmaf_rn(lvl, s, o);
-                if (mq) v = __fadd_rn(v, __fmul_rn(msc, (float)mq[j]));
-                dequant[dst + j] = v;
+    if (warp == 0 && lane < ns) {
+        s_s[lane] = __half2float(__ushort_as_half((unsigned short)(byte(0) | (byte(1) << 8))));
+        s_o[lane] = __half2float(__ushort_as_half((unsigned short)(byte(2) | (byte(3) << 8))));
+        x = dyn[32 + lane];
+    }
+    for (int k = 0; k <= T.hs; ++k) {
+        if (warp == 0) {
+            if (k < T.hs && lane < ns)
+#pragma unroll 1
+                for (int j = 0; j < (PAIR ? 16 : 32); ++j)
+                    tile[k & 1][lane * kSymRow + j] = decode4(lut, x, ptr, T.rec, 1u << 23, window);
+        } else if (k > 0) {
+#pragma unroll 4
+            for (int i = warp - 1; i < ns; i += kExportWarps - 1) {
+                const int h = s_grp[i] * T.hs + k - 1;
+                const unsigned long long mi = s_mi[i] == kNoMean ? kNoMean : s_mi[i] + h;
+                write_row<PAIR>(a, tile[(k - 1) & 1] + i * kSymRow, ((size_t)s_t[i] * a.Hkv + h) * DQ_HEAD_DIM, mi != kNoMean,
+                                load_mean(a, mi, lane), s_s[i], s_o[i], lane);
             }
-        };
-        if (T.pair) {   // one step per pair of values: entry = code(b) << 24 | f << 16 | code(a) << 8 | (z - c)
-            for (int j = 0; j < DQ_HEAD_DIM; j += 2) {
-                const uint32_t e = T.lut[x & 255u];
-                x = ((e >> 16) & 255u) * (x >> 8) + (e & 255u);
-                if (x < (1u << 23) && ptr < T.rec) x = (x << 8) | byte_at(ptr++);
-                emit(j, __half2float(__ushort_as_half((unsigned short)(e & 0xff00u))));
-                emit(j + 1, __half2float(__ushort_as_half((unsigned short)((e >> 16) & 0xff00u))));
-            }
-            continue;
         }
-        for (int j = 0; j < DQ_HEAD_DIM; ++j) {
-            const uint32_t e = T.lut[x & 255u];
-            x = (e >> 24) * (x >> 8) + (e & 255u);
-            if (x < (1u << 23) && ptr < T.rec) x = (x << 8) | byte_at(ptr++);
-            emit(j, __half2float(__ushort_as_half((unsigned short)((e >> 8) & 0xffffu))));
-        }
+        __syncthreads();
     }
 }
 
@@ -150,16 +281,19 @@ cudaError_t dq_launch_decode_tokens(const DqDevTable& t, const uint8_t* cont, co
                                     const float* mean_scale, int max_windows, const int32_t* seq_id,
                                     const int32_t* pos, const int32_t* slot, int T, int Hkv,
                                     uint8_t* symbols, float* dequant, cudaStream_t st) {
+    const ExportArgs a{cont, mean_q, mean_scale, seq_id, pos, slot, symbols, dequant, max_windows, T, Hkv};
     if (t.hs > 1) {
         const long long ns = (long long)T * (Hkv / t.hs);
         if (ns == 0) return cudaSuccess;
-        dq_decode_tokens_wide_kernel<<<(unsigned)((ns + 127) / 128), 128, 0, st>>>(
-            t, cont, mean_q, mean_scale, max_windows, seq_id, pos, slot, T, Hkv, symbols, dequant);
+        auto kernel = t.pair ? dq_decode_tokens_wide_kernel<true> : dq_decode_tokens_wide_kernel<false>;
+        const int smem = t.rec_words * 128;   // at most 32 KB
+        kernel<<<(unsigned)((ns + 31) / 32), kExportWarps * 32, smem, st>>>(t, a);
         return cudaGetLastError();
     }
     const long long n = (long long)T * Hkv;
     if (n == 0) return cudaSuccess;
-    dq_decode_tokens_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
-        t, cont, mean_q, mean_scale, max_windows, seq_id, pos, slot, T, Hkv, symbols, dequant);
+    auto kernel = t.pair ? dq_decode_tokens_kernel<true> : dq_decode_tokens_kernel<false>;
+    const int smem = kExportWarps * 32 * ((((t.rec + 10) >> 2) | 1) + kSymRow) * 4;   // at most 39 KB
+    kernel<<<(unsigned)((n + kExportWarps * 32 - 1) / (kExportWarps * 32)), kExportWarps * 32, smem, st>>>(t, a);
     return cudaGetLastError();
 }
