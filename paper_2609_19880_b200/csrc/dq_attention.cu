@@ -1148,7 +1148,10 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
     const int G1 = a.Hq / a.Hkv, G = G1 * q_len;   // rows per KV head
     const bool wide = tk.hs > 1;   // token-wide streams: main kernel of dq_attention_wide.cu
     Layout L = make_layout(nw, tk.rec, tv.rec, a.B, G);
-    if (wide) {
+    const int small = wide ? 0 : dq_attn_small_pick_warps(tk, tv, a.B, a.Hkv, a.max_pages, sm_count, smem_max);
+    if (small) {
+        nw = small;
+    } else if (wide) {
         nw = dq_attn_wide_pick_warps(tk, tv, a.B, G, smem_max);
         if (nw == 0) return cudaErrorInvalidConfiguration;
     } else {
@@ -1181,7 +1184,7 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
     // Decode-step mode pays (dynamic item order, late wait) while the encoder's ~20 us matter: not when every
     // CTA has dozens of items anyway (upper bound from the page-table width; the lengths live on the device).
     const long long max_items = (long long)a.B * ((a.max_pages * DQ_PAGE_TOKENS + nw * kChunk - 1) / (nw * kChunk)) * a.Hkv;
-    p.fused = a.fused && !wide && max_items <= 32LL * sm_count; p.attn_grid = sm_count; p.flags = p.counter;
+    p.fused = a.fused && !wide && !small && max_items <= 32LL * sm_count; p.attn_grid = sm_count; p.flags = p.counter;
     p.poll_limit = p.fused ? step_poll_limit() : 0;
     p.ne_before = p.prefix + (a.B + 1);
     p.item_tokens = nw * kChunk;
@@ -1194,6 +1197,20 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
     p.resid_lens = a.resid_lens; p.resid_cap = a.resid_cap;
 
     const int heads = a.B * a.Hq * q_len;
+    const bool prof = g_prof_on && g_prof_count < kProfRing && (g_prof_calls++ % g_prof_period) == 0;
+    if (prof && !g_prof_made[g_prof_count]) {
+        cudaError_t e;
+        if ((e = cudaEventCreate(&g_prof_ev[g_prof_count][0])) != cudaSuccess) return e;
+        if ((e = cudaEventCreate(&g_prof_ev[g_prof_count][1])) != cudaSuccess) return e;
+        g_prof_made[g_prof_count] = true;
+    }
+    if (small) {
+        if (prof) cudaEventRecord(g_prof_ev[g_prof_count][0], st);
+        const cudaError_t e = dq_launch_attention_small(tk, tv, p, nw, a.fused != 0, st);
+        if (e != cudaSuccess) return e;
+        if (prof) cudaEventRecord(g_prof_ev[g_prof_count++][1], st);
+        return dq_launch_pdl(dq_attn_combine_kernel, dim3(heads), dim3(256), 0, st, p);
+    }
     const long long prep_warps = (long long)heads * (1 + (p.has_mean ? (p.windows + kPrepWindows - 1) / kPrepWindows : 0));
     cudaError_t e = dq_launch_pdl(dq_attn_prepare_kernel, dim3((unsigned)((prep_warps + 7) / 8)), dim3(256), 0, st, p);
     if (e != cudaSuccess) return e;
@@ -1207,15 +1224,7 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
         e = cudaFuncSetAttribute(main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
         if (e != cudaSuccess) return e;
     }
-    const bool prof = g_prof_on && g_prof_count < kProfRing && (g_prof_calls++ % g_prof_period) == 0;
-    if (prof) {
-        if (!g_prof_made[g_prof_count]) {
-            if ((e = cudaEventCreate(&g_prof_ev[g_prof_count][0])) != cudaSuccess) return e;
-            if ((e = cudaEventCreate(&g_prof_ev[g_prof_count][1])) != cudaSuccess) return e;
-            g_prof_made[g_prof_count] = true;
-        }
-        cudaEventRecord(g_prof_ev[g_prof_count][0], st);
-    }
+    if (prof) cudaEventRecord(g_prof_ev[g_prof_count][0], st);
     if (wide) e = dq_launch_attention_wide_main(tk, tv, p, nw, sm_count, st);
     else e = dq_launch_pdl(main_kernel, dim3(sm_count), dim3(nw * 32), (size_t)L.total, st, tk, tv, p);
     if (e != cudaSuccess) return e;

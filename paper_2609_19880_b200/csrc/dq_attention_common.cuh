@@ -100,3 +100,9 @@ __device__ __forceinline__ int row_offset(const AttnParams& p, int r) {
 int dq_attn_wide_pick_warps(const DqDevTable& tk, const DqDevTable& tv, int B, int G, int smem_max);
 cudaError_t dq_launch_attention_wide_main(const DqDevTable& tk, const DqDevTable& tv, const dqattn::AttnParams& p,
                                           int nw, int sm_count, cudaStream_t st);
+
+// Calls whose blocks fit the GPU once (dq_attention_small.cu): warps per CTA (0: not such a call), and the launch,
+// which needs no prepare kernel.
+int dq_attn_small_pick_warps(const DqDevTable& tk, const DqDevTable& tv, int B, int Hkv, int max_pages, int sm_count, int smem_max);
+cudaError_t dq_launch_attention_small(const DqDevTable& tk, const DqDevTable& tv, const dqattn::AttnParams& p, int nw, bool step,
+                                      cudaStream_t st);
