@@ -20,7 +20,7 @@ _SOURCES = [
     ("dq_decode_tokens.cu", []),
     ("dq_attention.cu", []),
     ("dq_attention_wide.cu", []),
-    ("dq_attention_small.cu", ["-Xptxas", "-O1"]),   # keeps the order of the interleaved decode chains
+    ("dq_attention_small.cu", []),   # keeps the order of the interleaved decode chains
     ("dq_microbench.cu", []),
     ("dq_encode.cu", ["-fmad=false"]),
     ("dq_encode_batch.cu", ["-fmad=false"]),

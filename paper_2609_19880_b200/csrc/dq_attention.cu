@@ -32,7 +32,7 @@ using namespace dqattn;
 
 namespace {
 
-constexpr int kTileStride = 48;        // bytes per token row of a [32 tok][16 ch] fp16 tile; the
+constexpr int kTileStride = 32;        // bytes per token row of a [32 tok][16 ch] fp16 tile; the
                                        // 16 pad bytes of the K tile rows hold (sK, oK, sV, oV)
 constexpr int kTileBytes = kChunk * kTileStride;
 constexpr int kKTail = 32;             // bytes after a warp's K records: q'.mean of its window, per head
@@ -268,8 +268,10 @@ __device__ __forceinline__ void fused_pass(uint32_t xk, uint32_t ptrk, uint32_t 
                                            uint32_t obuf, int lane, int G, float (&sacc)[4][4],
                                            const uint32_t (&pb_hi)[2][2], const uint32_t (&pb_lo)[2][2]) {
     const uint32_t a_addr = q16 + ((lane & 7) + ((lane >> 3) & 1) * 8) * kQ16Stride + (lane >> 4) * 16;
-    const uint32_t bk_addr = ktile + ((lane & 7) + (lane >> 4) * 8) * kTileStride + ((lane >> 3) & 1) * 16;
-    const uint32_t av_addr = vtile + ((lane & 7) + (lane >> 4) * 8) * kTileStride + ((lane >> 3) & 1) * 16;
+    const int lrow = (lane & 7) + (lane >> 4) * 8;
+    const uint32_t ld_off = lrow * 32 + ((((lane >> 3) & 1) ^ ((lrow >> 2) & 1)) << 4);
+    const uint32_t bk_addr = ktile + ld_off, av_addr = vtile + ld_off;
+    const uint32_t st_lo = lane * 32 + (((lane >> 2) & 1) << 4), st_hi = lane * 32 + ((((lane >> 2) & 1) ^ 1) << 4);
     // output slot: thread holds channels (lane/4, lane/4 + 8) of heads (2 qd, 2 qd + 1)
     const uint32_t o_addr = obuf + ((2 * (lane & 3)) * kORow + (lane >> 2)) * 4;
 #ifndef DQ_EXP_CG
@@ -280,8 +282,8 @@ __device__ __forceinline__ void fused_pass(uint32_t xk, uint32_t ptrk, uint32_t 
         uint32_t pk[8], pv[8];
         if (DO_K) { if (PAIRS) decode16_pairs<LBITS>(xk, ptrk, lutk, one, pk); else decode16<LBITS>(xk, ptrk, lutk, one, pk); }
         if (DO_V) { if (PAIRS) decode16_pairs<LBITS>(xv, ptrv, lutv, one, pv); else decode16<LBITS>(xv, ptrv, lutv, one, pv); }
-        if (DO_K) { sts128(ktile + lane * kTileStride, pk); sts128(ktile + lane * kTileStride + 16, pk + 4); }
-        if (DO_V) { sts128(vtile + lane * kTileStride, pv); sts128(vtile + lane * kTileStride + 16, pv + 4); }
+        if (DO_K) { sts128(ktile + st_lo, pk); sts128(ktile + st_hi, pk + 4); }
+        if (DO_V) { sts128(vtile + st_lo, pv); sts128(vtile + st_hi, pv + 4); }
         __syncwarp();
         if (DO_K) {
             uint32_t a[4], b0[4], b1[4];
@@ -583,7 +585,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                 const float sV = __half2float(__ushort_as_half((unsigned short)(hv & 0xffffu)));
                 const float oV = __half2float(__ushort_as_half((unsigned short)(hv >> 16)));
                 // the key scale carries the logit scale (sm_scale * log2 e): logits come out in base-2 units
-                asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};\n" ::"r"(ktile + lane * kTileStride + 32),
+                asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};\n" ::"r"(ktile + lane * 16),
                              "f"(sK * p.scale_log2), "f"(oK), "f"(sV), "f"(oV) : "memory");
             }
             // tokens this thread's row may see: a query token that is not the last one stops earlier; tokens
@@ -597,7 +599,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
             }
             __syncwarp();
             float mx = -INFINITY;
-            const uint32_t meta = ktile + 2 * qd * kTileStride + 32;
+            const uint32_t meta = ktile + 2 * qd * 16;
             if (tok0 + kChunk <= row_len) {   // every token of the chunk is visible: no masks
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -605,7 +607,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                     for (int u = 0; u < 2; ++u) {
                         float4 m4;
                         asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-                                     : "=f"(m4.x), "=f"(m4.y), "=f"(m4.z), "=f"(m4.w) : "r"(meta + (8 * i + u) * kTileStride));
+                                     : "=f"(m4.x), "=f"(m4.y), "=f"(m4.z), "=f"(m4.w) : "r"(meta + (8 * i + u) * 16));
                         lg[i][u] = fmaf(m4.x, sacc[i][u] + sacc[i][2 + u], fmaf(m4.y, qs, qmu));
                         sv_t[i][u] = m4.z;
                         ov_t[i][u] = m4.w;
@@ -619,7 +621,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                     for (int u = 0; u < 2; ++u) {
                         float4 m4;
                         asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-                                     : "=f"(m4.x), "=f"(m4.y), "=f"(m4.z), "=f"(m4.w) : "r"(meta + (8 * i + u) * kTileStride));
+                                     : "=f"(m4.x), "=f"(m4.y), "=f"(m4.z), "=f"(m4.w) : "r"(meta + (8 * i + u) * 16));
                         const bool ok = 8 * i + u < lim;
                         lg[i][u] = ok ? fmaf(m4.x, sacc[i][u] + sacc[i][2 + u], fmaf(m4.y, qs, qmu)) : -INFINITY;
                         sv_t[i][u] = ok ? m4.z : 0.f;

@@ -58,10 +58,10 @@ __device__ __forceinline__ void step_both(uint32_t (&x)[2], uint32_t (&sel)[2], 
         : "+r"(x[0]), "+r"(x[1]), "+r"(sel[0]), "+r"(sel[1]) : "r"(win[0]), "r"(win[1]), "r"(one), "n"(1u << LBITS));
 }
 
-// 16 channels of both streams: levels as 8 fp16x2 words each.
+// 16 channels of both streams: levels as 8 fp16x2 words each into the lane's tile rows (halves swapped by `swap`).
 template <int LBITS, bool PAIRS>
 __device__ __forceinline__ void decode16_both(uint32_t (&x)[2], uint32_t (&ptr)[2], const uint32_t (&lut)[2], uint32_t one,
-                                              uint32_t (&pk)[8], uint32_t (&pv)[8]) {
+                                              uint32_t krow, uint32_t vrow, uint32_t swap) {
 #pragma unroll
     for (int q4 = 0; q4 < (PAIRS ? 2 : 4); ++q4) {
         uint32_t sel[2] = {0x2104u, 0x2104u}, win[2], lo[2], hi[2];
@@ -74,12 +74,16 @@ __device__ __forceinline__ void decode16_both(uint32_t (&x)[2], uint32_t (&ptr)[
         for (int i = 0; i < 4; ++i) step_both<LBITS, PAIRS ? 0x00010000u : 0x01000000u>(x, sel, win, lut, one, e[i], d[i]);
         ptr[0] += sel[0] - 0x2104u;
         ptr[1] += sel[1] - 0x2104u;
+        // stored group by group: the stores keep the two chains' steps interleaved in the generated code
         if (PAIRS) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { pk[4 * q4 + i] = e[i] & 0xff00ff00u; pv[4 * q4 + i] = d[i] & 0xff00ff00u; }
+            const uint32_t k4[4] = {e[0] & 0xff00ff00u, e[1] & 0xff00ff00u, e[2] & 0xff00ff00u, e[3] & 0xff00ff00u};
+            const uint32_t v4[4] = {d[0] & 0xff00ff00u, d[1] & 0xff00ff00u, d[2] & 0xff00ff00u, d[3] & 0xff00ff00u};
+            sts128(krow + ((16u * q4) ^ swap), k4);
+            sts128(vrow + ((16u * q4) ^ swap), v4);
         } else {
-            pk[2 * q4] = __byte_perm(e[0], e[1], 0x6521u); pk[2 * q4 + 1] = __byte_perm(e[2], e[3], 0x6521u);
-            pv[2 * q4] = __byte_perm(d[0], d[1], 0x6521u); pv[2 * q4 + 1] = __byte_perm(d[2], d[3], 0x6521u);
+            const uint32_t at = ((16u * (q4 >> 1)) ^ swap) + 8u * (q4 & 1);
+            sts64(krow + at, __byte_perm(e[0], e[1], 0x6521u), __byte_perm(e[2], e[3], 0x6521u));
+            sts64(vrow + at, __byte_perm(d[0], d[1], 0x6521u), __byte_perm(d[2], d[3], 0x6521u));
         }
     }
 }
@@ -224,13 +228,10 @@ dq_attention_small_kernel(const __grid_constant__ DqDevTable TK, const __grid_co
         const uint32_t lut[2] = {sbase + kOffLutK + lane * 4, sbase + kOffLutV + lane * 4};
         const uint32_t one = (sbase >> 31) | 1u;
         const uint32_t a_addr = sbase + kOffQ16 + ((lane & 7) + ((lane >> 3) & 1) * 8) * kQ16Stride + (lane >> 4) * 16;
-        const uint32_t st_lo = lane * 32 + (((lane >> 2) & 1) << 4), st_hi = lane * 32 + ((((lane >> 2) & 1) ^ 1) << 4);
+        const uint32_t swap = ((lane >> 2) & 1) << 4;
 #pragma unroll 1
         for (int cg = 0; cg < 8; ++cg) {
-            uint32_t pk[8], pv[8];
-            decode16_both<LBITS, PAIRS>(x, ptr, lut, one, pk, pv);
-            sts128(ktile + st_lo, pk); sts128(ktile + st_hi, pk + 4);
-            sts128(vtiles + cg * kTile + st_lo, pv); sts128(vtiles + cg * kTile + st_hi, pv + 4);
+            decode16_both<LBITS, PAIRS>(x, ptr, lut, one, ktile + lane * 32, vtiles + cg * kTile + lane * 32, swap);
             __syncwarp();
             uint32_t a[4], b0[4], b1[4];
             ldmatrix_x4(a, a_addr + cg * 32);
