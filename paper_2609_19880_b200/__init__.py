@@ -127,13 +127,26 @@ def _check(rc, what):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()   # ctypes turns the integer into the void* of the argtypes
+
+
+_current_raw_stream = None
 
 
 def _stream(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    """cudaStream_t of ``stream``, or of the current stream (the raw lookup: building a Stream object takes 3 us)."""
+    global _current_raw_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_raw_stream is None:
+        import torch
+        try:
+            get, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+            _current_raw_stream = lambda: get(device())
+        except AttributeError:
+            _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        torch.cuda.init()
+    return _current_raw_stream()
 
 
 class Tables:
@@ -186,7 +199,7 @@ def dq_encode_tokens(tk, tv, k_bf16, v_bf16, seq_id, pos, slot, k_cont, v_cont, 
     rope = (cos f32 [positions, 64], sin, style): keys are given before their rotary embedding."""
     ref = k_bf16 if k_bf16 is not None else v_bf16
     T, Hkv = int(ref.shape[0]), int(ref.shape[1])
-    max_windows = int(k_mean_q.shape[1]) if k_mean_q is not None else 0
+    max_windows = k_mean_q.shape[1] if k_mean_q is not None else 0
     common = (tk.handle if tk else None, tv.handle if tv else None, _ptr(k_bf16), _ptr(v_bf16),
               T, Hkv, _ptr(seq_id), _ptr(pos), _ptr(slot), _ptr(k_cont), _ptr(v_cont),
               _ptr(k_mean_q), _ptr(k_mean_scale), max_windows, int(mean_mode))
@@ -205,12 +218,12 @@ def dq_decode_workspace_bytes(B: int, Hq: int, max_pages: int) -> int:
 def dq_decode_attention(tk, tv, q_bf16, k_cont, v_cont, k_mean_q, k_mean_scale, page_table, seq_lens,
                         Hkv: int, sm_scale: float, out_bf16, workspace, out_f32=None, stream=None):
     """q bf16 [B, Hq, 128], containers, seq_lens -> out bf16 [B, Hq, 128]."""
-    B, Hq = int(q_bf16.shape[0]), int(q_bf16.shape[1])
-    max_windows = int(k_mean_q.shape[1]) if k_mean_q is not None else 0
+    B, Hq = q_bf16.shape[:2]
+    max_windows = k_mean_q.shape[1] if k_mean_q is not None else 0
     rc = lib().dq_decode_attention(tk.handle, tv.handle, _ptr(q_bf16), _ptr(k_cont), _ptr(v_cont), _ptr(k_mean_q),
-                                   _ptr(k_mean_scale), max_windows, _ptr(page_table), int(page_table.shape[1]),
+                                   _ptr(k_mean_scale), max_windows, _ptr(page_table), page_table.shape[1],
                                    _ptr(seq_lens), B, Hq, int(Hkv), float(sm_scale), _ptr(out_bf16),
-                                   _ptr(out_f32), _ptr(workspace), int(workspace.numel() * workspace.element_size()),
+                                   _ptr(out_f32), _ptr(workspace), workspace.nbytes,
                                    _stream(stream))
     _check(rc, "dq_decode_attention")
 
@@ -220,13 +233,13 @@ def dq_decode_attention_residual(tk, tv, q_bf16, k_cont, v_cont, k_mean_q, k_mea
                                  out_f32=None, stream=None):
     """Decode attention over the compressed cache plus a BF16 residual window:
     resid_k / resid_v bf16 [B, cap, Hkv, 128], resid_lens int32 [B]."""
-    B, Hq = int(q_bf16.shape[0]), int(q_bf16.shape[1])
-    max_windows = int(k_mean_q.shape[1]) if k_mean_q is not None else 0
+    B, Hq = q_bf16.shape[:2]
+    max_windows = k_mean_q.shape[1] if k_mean_q is not None else 0
     rc = lib().dq_decode_attention_residual(
         tk.handle, tv.handle, _ptr(q_bf16), _ptr(k_cont), _ptr(v_cont), _ptr(k_mean_q), _ptr(k_mean_scale),
-        max_windows, _ptr(page_table), int(page_table.shape[1]), _ptr(seq_lens), _ptr(resid_k), _ptr(resid_v),
+        max_windows, _ptr(page_table), page_table.shape[1], _ptr(seq_lens), _ptr(resid_k), _ptr(resid_v),
         _ptr(resid_lens), int(resid_k.shape[1]), B, Hq, int(Hkv), float(sm_scale), _ptr(out_bf16), _ptr(out_f32),
-        _ptr(workspace), int(workspace.numel() * workspace.element_size()), _stream(stream))
+        _ptr(workspace), workspace.nbytes, _stream(stream))
     _check(rc, "dq_decode_attention_residual")
 
 
@@ -235,13 +248,13 @@ def dq_decode_attention_multi(tk, tv, q_bf16, k_cont, v_cont, k_mean_q, k_mean_s
                               resid_v=None, resid_lens=None, stream=None):
     """q bf16 [B, q_len, Hq, 128] -> out bf16 [B, q_len, Hq, 128]: q_len query tokens per sequence share
     one pass over the cache; seq_lens (+ resid_lens) include the q_len newest tokens."""
-    B, q_len, Hq = int(q_bf16.shape[0]), int(q_bf16.shape[1]), int(q_bf16.shape[2])
-    max_windows = int(k_mean_q.shape[1]) if k_mean_q is not None else 0
+    B, q_len, Hq = q_bf16.shape[:3]
+    max_windows = k_mean_q.shape[1] if k_mean_q is not None else 0
     rc = lib().dq_decode_attention_multi(
         tk.handle, tv.handle, _ptr(q_bf16), q_len, _ptr(k_cont), _ptr(v_cont), _ptr(k_mean_q), _ptr(k_mean_scale),
-        max_windows, _ptr(page_table), int(page_table.shape[1]), _ptr(seq_lens), _ptr(resid_k), _ptr(resid_v),
+        max_windows, _ptr(page_table), page_table.shape[1], _ptr(seq_lens), _ptr(resid_k), _ptr(resid_v),
         _ptr(resid_lens), int(resid_k.shape[1]) if resid_k is not None else 0, B, Hq, int(Hkv), float(sm_scale),
-        _ptr(out_bf16), _ptr(out_f32), _ptr(workspace), int(workspace.numel() * workspace.element_size()),
+        _ptr(out_bf16), _ptr(out_f32), _ptr(workspace), workspace.nbytes,
         _stream(stream))
     _check(rc, "dq_decode_attention_multi")
 
@@ -250,13 +263,13 @@ def dq_decode_step(tk, tv, k_new, v_new, slot_new, q_bf16, k_cont, v_cont, k_mea
                    seq_lens, Hkv: int, sm_scale: float, out_bf16, workspace, out_f32=None, status=None, stream=None):
     """Encode the newest token of every sequence (k_new / v_new bf16 [B, Hkv, 128] at slot_new, position
     seq_lens - 1) and attend over the whole cache, as one overlapped launch sequence."""
-    B, Hq = int(q_bf16.shape[0]), int(q_bf16.shape[1])
-    max_windows = int(k_mean_q.shape[1]) if k_mean_q is not None else 0
+    B, Hq = q_bf16.shape[:2]
+    max_windows = k_mean_q.shape[1] if k_mean_q is not None else 0
     rc = lib().dq_decode_step(tk.handle, tv.handle, _ptr(k_new), _ptr(v_new), _ptr(slot_new), _ptr(q_bf16),
                               _ptr(k_cont), _ptr(v_cont), _ptr(k_mean_q), _ptr(k_mean_scale), max_windows,
-                              _ptr(page_table), int(page_table.shape[1]), _ptr(seq_lens), B, Hq, int(Hkv),
+                              _ptr(page_table), page_table.shape[1], _ptr(seq_lens), B, Hq, int(Hkv),
                               float(sm_scale), _ptr(out_bf16), _ptr(out_f32), _ptr(workspace),
-                              int(workspace.numel() * workspace.element_size()), _ptr(status), _stream(stream))
+                              workspace.nbytes, _ptr(status), _stream(stream))
     _check(rc, "dq_decode_step")
 
 
@@ -276,11 +289,11 @@ def dq_decode_attention_static(tk, tv, q_bf16, k_cont, v_cont, k_mean_q, k_mean_
     scratch array (STATIC_SCRATCH_BYTES, shared by all calls) is used instead.  Raises
     DqError(DQ_ERR_WORKSPACE) when the call would need more than that.  Calls must not overlap
     on the GPU; make the first call on a device outside any stream capture."""
-    B, Hq = int(q_bf16.shape[0]), int(q_bf16.shape[1])
-    max_windows = int(k_mean_q.shape[1]) if k_mean_q is not None else 0
+    B, Hq = q_bf16.shape[:2]
+    max_windows = k_mean_q.shape[1] if k_mean_q is not None else 0
     rc = lib().dq_decode_attention_static(tk.handle, tv.handle, _ptr(q_bf16), _ptr(k_cont), _ptr(v_cont),
                                           _ptr(k_mean_q), _ptr(k_mean_scale), max_windows, _ptr(page_table),
-                                          int(page_table.shape[1]), _ptr(seq_lens), B, Hq, int(Hkv),
+                                          page_table.shape[1], _ptr(seq_lens), B, Hq, int(Hkv),
                                           float(sm_scale), _ptr(out_bf16), _ptr(out_f32), _stream(stream))
     if rc == -4:
         raise DqError(rc, "dq_decode_attention_static [" + lib().dq_last_cuda_error().decode() + "]")
@@ -289,7 +302,7 @@ def dq_decode_attention_static(tk, tv, q_bf16, k_cont, v_cont, k_mean_q, k_mean_
 
 def dq_decode_tokens(t, cont, slot, Hkv: int, symbols=None, dequant=None, mean_q=None, mean_scale=None,
                      seq_id=None, pos=None, stream=None):
-    max_windows = int(mean_q.shape[1]) if mean_q is not None else 0
+    max_windows = mean_q.shape[1] if mean_q is not None else 0
     rc = lib().dq_decode_tokens(t.handle, _ptr(cont), _ptr(mean_q), _ptr(mean_scale), max_windows, _ptr(seq_id),
                                 _ptr(pos), _ptr(slot), int(slot.shape[0]), int(Hkv), _ptr(symbols), _ptr(dequant),
                                 _stream(stream))
@@ -298,11 +311,11 @@ def dq_decode_tokens(t, cont, slot, Hkv: int, symbols=None, dequant=None, mean_q
 
 def dq_bf16_decode_attention(q_bf16, k_pages, v_pages, page_table, seq_lens, Hkv: int, sm_scale: float,
                              out_bf16, workspace, stream=None):
-    B, Hq = int(q_bf16.shape[0]), int(q_bf16.shape[1])
+    B, Hq = q_bf16.shape[:2]
     rc = lib().dq_bf16_decode_attention(_ptr(q_bf16), _ptr(k_pages), _ptr(v_pages), _ptr(page_table),
-                                        int(page_table.shape[1]), _ptr(seq_lens), B, Hq, int(Hkv), float(sm_scale),
+                                        page_table.shape[1], _ptr(seq_lens), B, Hq, int(Hkv), float(sm_scale),
                                         _ptr(out_bf16), _ptr(workspace),
-                                        int(workspace.numel() * workspace.element_size()), _stream(stream))
+                                        workspace.nbytes, _stream(stream))
     _check(rc, "dq_bf16_decode_attention")
 
 

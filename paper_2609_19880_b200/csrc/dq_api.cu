@@ -54,6 +54,31 @@ long long dq_opt_encode_batch_min(long long dflt) {
     return v < 0 ? dflt : v;
 }
 
+// Largest dynamic shared memory already granted, by (kernel, device); a slot is claimed once and never moves.
+cudaError_t dq_allow_smem(const void* kernel, int bytes) {
+    constexpr int kSlots = 512, kDevs = 16;
+    struct Slot {
+        std::atomic<const void*> kernel{nullptr};
+        std::atomic<int> granted[kDevs] = {};
+    };
+    static Slot slots[kSlots];
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::atomic<int>* granted = nullptr;
+    if (dev < kDevs) {
+        unsigned at = (unsigned)((reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u) % kSlots;
+        for (int probe = 0; probe < kSlots && !granted; ++probe, at = (at + 1) % kSlots) {
+            const void* seen = nullptr;
+            if (slots[at].kernel.compare_exchange_strong(seen, kernel) || seen == kernel) granted = &slots[at].granted[dev];
+        }
+        if (granted && granted->load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    }
+    const cudaError_t set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (set == cudaSuccess && granted) granted->store(bytes, std::memory_order_release);
+    return set;
+}
+
 extern "C" {
 
 int dq_build_tables(int levels, double bits_per_elem, const dq_table_opts* opts, dq_tables** out) {

@@ -1154,7 +1154,7 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
     if (small) {
         nw = small;
     } else if (wide) {
-        nw = dq_attn_wide_pick_warps(tk, tv, a.B, G, smem_max);
+        nw = dq_attn_wide_pick_warps(tk, tv, a.B, G, a.Hkv / tk.hs, a.max_pages, sm_count, smem_max);
         if (nw == 0) return cudaErrorInvalidConfiguration;
     } else {
         while (L.total > smem_max && nw > 4) {
@@ -1223,7 +1223,7 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
                 : (tk.sigma == 24 ? (p.fused ? dq_attention_kernel<true, 15, false> : dq_attention_kernel<false, 15, false>)
                                   : (p.fused ? dq_attention_kernel<true, 23, false> : dq_attention_kernel<false, 23, false>));
     if (!wide) {
-        e = cudaFuncSetAttribute(main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+        e = dq_allow_smem(reinterpret_cast<const void*>(main_kernel), L.total);
         if (e != cudaSuccess) return e;
     }
     if (prof) cudaEventRecord(g_prof_ev[g_prof_count][0], st);
@@ -1291,7 +1291,7 @@ cudaError_t dq_launch_bf16_attention(const DqAttnArgs& a, const void* k_pages, c
     cudaError_t e = device_limits(&sm_count, &smem_max);
     if (e != cudaSuccess) return e;
     if (kBfSmem + 17 * 1024 > smem_max) return cudaErrorInvalidConfiguration;   // ring + the static scan arrays
-    e = cudaFuncSetAttribute(dq_bf16_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBfSmem);
+    e = dq_allow_smem(reinterpret_cast<const void*>(dq_bf16_attention_kernel), kBfSmem);
     if (e != cudaSuccess) return e;
     e = dq_launch_pdl(dq_bf16_attention_kernel, dim3(sm_count), dim3(kBfWarps * 32), (size_t)kBfSmem, st, p,
                       static_cast<const uint16_t*>(k_pages), static_cast<const uint16_t*>(v_pages),

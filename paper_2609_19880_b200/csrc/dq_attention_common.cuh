@@ -100,7 +100,7 @@ __device__ __forceinline__ int row_offset(const AttnParams& p, int r) {
 
 // Main kernel of the token-wide path (dq_attention_wide.cu): warps per CTA that fit the
 // device's shared memory (0: none do), and the launch itself; prepare / combine are shared.
-int dq_attn_wide_pick_warps(const DqDevTable& tk, const DqDevTable& tv, int B, int G, int smem_max);
+int dq_attn_wide_pick_warps(const DqDevTable& tk, const DqDevTable& tv, int B, int G, int groups, int max_pages, int sm_count, int smem_max);
 cudaError_t dq_launch_attention_wide_main(const DqDevTable& tk, const DqDevTable& tv, const dqattn::AttnParams& p,
                                           int nw, int sm_count, cudaStream_t st);
 

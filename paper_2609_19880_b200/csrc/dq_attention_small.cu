@@ -388,7 +388,7 @@ cudaError_t dq_launch_attention_small(const DqDevTable& tk, const DqDevTable& tv
                 : (tk.sigma == 24 ? (step ? dq_attention_small_kernel<true, 15, false> : dq_attention_small_kernel<false, 15, false>)
                                   : (step ? dq_attention_small_kernel<true, 23, false> : dq_attention_small_kernel<false, 23, false>));
     const int smem = small_smem_bytes(nw, tk.rec, tv.rec, p.B);
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = dq_allow_smem(reinterpret_cast<const void*>(kernel), smem);
     if (e != cudaSuccess) return e;
     const int blocks = p.B * ((p.max_pages * DQ_PAGE_TOKENS + nw * kChunk - 1) / (nw * kChunk)) * p.Hkv;
     return dq_launch_pdl(kernel, dim3((unsigned)blocks), dim3(nw * 32), (size_t)smem, st, tk, tv, p);

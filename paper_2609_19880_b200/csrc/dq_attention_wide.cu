@@ -115,6 +115,50 @@ __device__ __forceinline__ void decode16_ring_pairs(uint32_t& x, uint32_t& ptr, 
     }
 }
 
+// Both streams of a lane, their steps in turn; a group of four steps goes to the tiles right away, which keeps the
+// two chains interleaved in the generated code (two chains then take little longer than one).
+template <bool PAIRS>
+__device__ __forceinline__ void decode16_rings(uint32_t& xk, uint32_t& ptrk, uint32_t ringk_lane, uint32_t lutk, uint32_t krow, uint32_t& xv,
+                                               uint32_t& ptrv, uint32_t ringv_lane, uint32_t lutv, uint32_t vrow, uint32_t swap,
+                                               uint32_t one) {
+    constexpr uint32_t FW = PAIRS ? 0x00010000u : 0x01000000u;
+    uint32_t x[2] = {xk, xv}, ptr[2] = {ptrk, ptrv};
+    const uint32_t lut[2] = {lutk, lutv}, ring[2] = {ringk_lane, ringv_lane};
+    constexpr uint32_t mask[2] = {(uint32_t)(kRowsK - 1) << 7, (uint32_t)(kRowsV - 1) << 7};
+#pragma unroll
+    for (int q4 = 0; q4 < (PAIRS ? 2 : 4); ++q4) {
+        uint32_t sel[2] = {0x2104u, 0x2104u}, win[2], e[2][4];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const uint32_t t = ptr[c] << 5;
+            win[c] = __funnelshift_r(lds32(ring[c] + (t & mask[c])), lds32(ring[c] + ((t + 128u) & mask[c])), ptr[c] << 3);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t f[2], t[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) e[c][i] = lds32(dp4a_u32(x[c], 0x80u, lut[c]));
+#pragma unroll
+            for (int c = 0; c < 2; ++c) { f[c] = dp4a_u32(e[c][i], FW, 0u); t[c] = f[c] * (x[c] >> 8); x[c] = dp4a_u32(e[c][i], 1u, t[c]); }
+            asm("{.reg .pred p, q; setp.lt.u32 p, %0, 0x800000; setp.lt.u32 q, %1, 0x800000; @p prmt.b32 %0, %0, %4, %2; "
+                "@q prmt.b32 %1, %1, %5, %3; @p mad.lo.u32 %2, %6, %6, %2; @q mad.lo.u32 %3, %6, %6, %3;}"
+                : "+r"(x[0]), "+r"(x[1]), "+r"(sel[0]), "+r"(sel[1]) : "r"(win[0]), "r"(win[1]), "r"(one));
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            ptr[c] += sel[c] - 0x2104u;
+            const uint32_t row = c ? vrow : krow;
+            if (PAIRS) {
+                const uint32_t w4[4] = {e[c][0] & 0xff00ff00u, e[c][1] & 0xff00ff00u, e[c][2] & 0xff00ff00u, e[c][3] & 0xff00ff00u};
+                sts128(row + ((16u * q4) ^ swap), w4);
+            } else {
+                sts64(row + ((16u * (q4 >> 1)) ^ swap) + 8u * (q4 & 1), __byte_perm(e[c][0], e[c][1], 0x6521u), __byte_perm(e[c][2], e[c][3], 0x6521u));
+            }
+        }
+    }
+    xk = x[0]; xv = x[1]; ptrk = ptr[0]; ptrv = ptr[1];
+}
+
 // The same 16 symbols for a warp in which some lane lags too far behind the ring: such a lane
 // (`fast` false) takes its window words from the record in global memory (col: its word 0;
 // consecutive words are 16 words apart).  Rare, kept out of line.
@@ -218,7 +262,11 @@ __device__ __forceinline__ void wide_pass(Chain& ck, Chain& cv, uint32_t ringk, 
         if (DO_V) fv = ring_advance<kRowsV>(cv, ringv_piece, v_cont, rwv, lane);
         cp_async_commit();
         uint32_t pk[8], pv[8];
-        if (__all_sync(kFullMask, fk && fv)) {
+        const bool fast = __all_sync(kFullMask, fk && fv);
+        if (fast && DO_K && DO_V) {
+            decode16_rings<PAIRS>(ck.x, ck.ptr, ringk_lane, lutk, ktile + lane * 32, cv.x, cv.ptr, ringv_lane, lutv, vtile + lane * 32, st_lo & 16u, one);
+        } else {
+        if (fast) {
             if (DO_K) { if (PAIRS) decode16_ring_pairs<kRowsK>(ck.x, ck.ptr, ringk_lane, lutk, one, pk); else decode16_ring<kRowsK>(ck.x, ck.ptr, ringk_lane, lutk, one, pk); }
             if (DO_V) { if (PAIRS) decode16_ring_pairs<kRowsV>(cv.x, cv.ptr, ringv_lane, lutv, one, pv); else decode16_ring<kRowsV>(cv.x, cv.ptr, ringv_lane, lutv, one, pv); }
         } else {   // some lane lags behind its ring: that lane reads global memory (rare, out of line)
@@ -239,6 +287,7 @@ __device__ __forceinline__ void wide_pass(Chain& ck, Chain& cv, uint32_t ringk, 
         }
         if (DO_K) { sts128(ktile + st_lo, pk); sts128(ktile + st_hi, pk + 4); }
         if (DO_V) { sts128(vtile + st_lo, pv); sts128(vtile + st_hi, pv + 4); }
+        }
         __syncwarp();
         if (DO_K) {
             uint32_t a[4], b0[4], b1[4];
@@ -593,18 +642,24 @@ dq_attention_wide_kernel(const __grid_constant__ DqDevTable TK, const __grid_con
 
 }  // namespace
 
-int dq_attn_wide_pick_warps(const DqDevTable& tk, const DqDevTable& tv, int B, int G, int smem_max) {
+// As many warps per CTA as the shared memory holds -- or the fewest with which the call's blocks (counted from the
+// width of the page table, the lengths being on the device) still fit the GPU once: the fewer warps share a scheduler,
+// the sooner a block's serial chains end.
+int dq_attn_wide_pick_warps(const DqDevTable& tk, const DqDevTable& tv, int B, int G, int groups, int max_pages, int sm_count, int smem_max) {
     (void)tk; (void)tv;
-    for (int nw = kWideWarps; nw >= 4; --nw)
-        if (wide_smem_bytes(nw, B, G) <= smem_max) return nw;
-    return 0;
+    int most = kWideWarps;
+    while (most >= 4 && wide_smem_bytes(most, B, G) > smem_max) --most;
+    if (most < 4) return 0;
+    for (int nw = 4; nw < most; ++nw)
+        if ((long long)B * ((max_pages * DQ_PAGE_TOKENS + nw * kChunk - 1) / (nw * kChunk)) * groups <= sm_count) return nw;
+    return most;
 }
 
 cudaError_t dq_launch_attention_wide_main(const DqDevTable& tk, const DqDevTable& tv, const AttnParams& p, int nw,
                                           int sm_count, cudaStream_t st) {
     const int smem_bytes = wide_smem_bytes(nw, p.B, p.G);
     auto kernel = tk.pair ? dq_attention_wide_kernel<true> : dq_attention_wide_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    cudaError_t e = dq_allow_smem(reinterpret_cast<const void*>(kernel), smem_bytes);
     if (e != cudaSuccess) return e;
     return dq_launch_pdl(kernel, dim3(sm_count), dim3(nw * 32), (size_t)smem_bytes, st, tk, tv, p);
 }

@@ -598,7 +598,7 @@ cudaError_t dq_launch_encode_wide(const DqDevTable& tk, const DqDevTable& tv, co
         const auto kernel = t.pair ? kernel_for<true>(t.M) : kernel_for<false>(t.M);
         if (!kernel) return cudaErrorInvalidValue;
         const int smem = wide_smem(t.hs, t.rec);
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = dq_allow_smem(reinterpret_cast<const void*>(kernel), smem);
         if (e != cudaSuccess) return e;
         e = dq_launch_pdl(kernel, dim3((unsigned)((streams + per - 1) / per)), dim3(t.hs * 32), (size_t)smem, st, t, kind == 0 ? pk : pv, a,
                           per, kind == 1, second);

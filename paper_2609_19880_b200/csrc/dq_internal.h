@@ -48,6 +48,10 @@ struct dq_tables {
 int dq_opt_step_poll_limit(int dflt);
 long long dq_opt_encode_batch_min(long long dflt);
 
+// dq_api.cu: lets `kernel` use `bytes` of dynamic shared memory on the current device (remembered: the runtime call
+// costs about as much as a tenth of a launch)
+cudaError_t dq_allow_smem(const void* kernel, int bytes);
+
 // dq_tables.cu
 int dq_host_build(int levels, double bits_per_elem, const dq_table_opts* opts, dq_tables* out);
 
