@@ -109,6 +109,11 @@ dq_attention_small_kernel(const __grid_constant__ DqDevTable TK, const __grid_co
     const uint32_t kst = wb + kWRec, vst = kst + align16s(kChunk * TK.rec);
 
     pdl_launch_dependents();
+    for (int i = tid; i < 256 * 8; i += nthreads) {   // tables (kernel parameters): 32 copies of an entry, 16 bytes at a time
+        const uint32_t k = TK.lut[i >> 3], v = TV.lut[i >> 3];
+        reinterpret_cast<uint4*>(lutk)[i] = make_uint4(k, k, k, k);
+        reinterpret_cast<uint4*>(lutv)[i] = make_uint4(v, v, v, v);
+    }
     // In decode-step mode the encoder let this kernel go after its own wait: everything older is complete, and only the
     // newest tokens' records and their windows' means are still being written.
     if (!STEP) pdl_wait_prior_grid();
@@ -134,12 +139,6 @@ dq_attention_small_kernel(const __grid_constant__ DqDevTable TK, const __grid_co
             carry += __shfl_sync(kFullMask, incl, 31);
         }
         if (lane == 0) { s_item[3] = carry; if (blockIdx.x == 0) p.prefix[p.B] = carry; }
-    } else {
-        for (int i = tid - 32; i < 256 * 8; i += nthreads - 32) {   // tables: a lane's column of 4-byte entries, 16 bytes at a time
-            const uint32_t k = TK.lut[i >> 3], v = TV.lut[i >> 3];
-            reinterpret_cast<uint4*>(lutk)[i] = make_uint4(k, k, k, k);
-            reinterpret_cast<uint4*>(lutv)[i] = make_uint4(v, v, v, v);
-        }
     }
     __syncthreads();
     const int bg = (int)blockIdx.x / p.Hkv, h = (int)blockIdx.x - bg * p.Hkv;
@@ -154,7 +153,14 @@ dq_attention_small_kernel(const __grid_constant__ DqDevTable TK, const __grid_co
     const bool mine = tok0 < len;   // this warp holds tokens
     if (STEP && late) pdl_wait_prior_grid();
 
-    // records of the warp's two pages
+    // the mean of the warp's window (used once q' is there) and the page ids of its 32 tokens
+    uint32_t q4 = 0u;
+    float msc = 0.f;
+    if (p.has_mean && mine) {
+        const size_t mi = ((size_t)b * p.max_windows + tok0 / DQ_WINDOW_TOKENS) * p.Hkv + h;
+        q4 = *reinterpret_cast<const uint32_t*>(p.mean_q + mi * kN + 4 * lane);
+        msc = p.mean_scale[mi];
+    }
     int page = 0;
     if (mine && lane < 2 && tok0 + 16 * lane < len) page = p.page_table[(size_t)b * p.max_pages + (tok0 >> 4) + lane];
     const int page0 = __shfl_sync(kFullMask, page, 0), page1 = __shfl_sync(kFullMask, page, 1);
@@ -195,9 +201,6 @@ dq_attention_small_kernel(const __grid_constant__ DqDevTable TK, const __grid_co
     }
     __syncthreads();
     if (p.has_mean && mine) {   // q'.mean of the warp's window, times the logit scale
-        const size_t mi = ((size_t)b * p.max_windows + tok0 / DQ_WINDOW_TOKENS) * p.Hkv + h;
-        const uint32_t q4 = *reinterpret_cast<const uint32_t*>(p.mean_q + mi * kN + 4 * lane);
-        const float msc = p.mean_scale[mi];
         float m[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) m[e] = msc * (float)(int)(int8_t)((q4 >> (8 * e)) & 0xffu);

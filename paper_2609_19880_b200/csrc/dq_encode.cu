@@ -194,7 +194,7 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
 
     const StreamQuantised sq = quantise_stream<PAIR>(T, a, is_v, t, h, lane);
     // rANS, Eq. (rans) Enc on symbols 127 .. 0 so that decoding runs forward.  Every lane
-    // carries the same state (the symbols come from shared memory); lane 0 records the bytes.
+    // carries the same state (the symbols come from shared memory).
     // (paired symbols: the lane's two pair indices u = a M + b; the coder then runs over 64 symbols)
     if (PAIR) {
         const uint32_t M = (uint32_t)T.M;
@@ -205,21 +205,10 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
     }
     __syncwarp();
     uint32_t xs = 1u << (T.sigma - 9);   // L: 2^23, or 2^15 with the 24-bit state
-    int k = 0;
-    // emitted bytes go to shared memory through stores the compiler does not treat as aliasing
-    // the symbol / table loads, so those loads are issued ahead of the serial state chain
     const uint32_t bytes_addr = dqdev::smem_addr(s_bytes[wib]);
-#pragma unroll 8
-    for (int j = (PAIR ? kN / 2 : kN) - 1; j >= 0; --j) {
-        const uint32_t m = s_sym[wib][j];
-        const uint4 en = T.enc[m];
-        if (xs >= en.y) {  // at most once: xs < 2^8 L <= 2^8 * (f L)
-            if (lane == 0) asm volatile("st.shared.u8 [%0], %1;" ::"r"(bytes_addr + k), "r"(xs & 0xffu));
-            ++k;
-            xs >>= 8;
-        }
-        xs = __funnelshift_r(__umulhi(xs, en.x), 0u, en.w) * (en.w >> 5) + (xs + en.z);
-    }
+    uint32_t dst = bytes_addr;           // every lane stores the same bytes to the same place
+    rans_encode_row<1>(T.enc, reinterpret_cast<const uint32_t*>(s_sym[wib]), (PAIR ? kN / 2 : kN) / 4, xs, dst);
+    const int k = (int)(dst - bytes_addr);
     __syncwarp();
     asm volatile("" ::: "memory");
     const uint32_t hdr0 = sq.hdr0;

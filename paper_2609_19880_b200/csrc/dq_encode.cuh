@@ -259,6 +259,26 @@ __device__ __forceinline__ void rans_step(uint32_t& x, uint32_t& dst, const uint
     x = __funnelshift_r(__umulhi(x, en.x), 0u, en.w) * (en.w >> 5) + (x + en.z);   // the shift uses en.w mod 32
 }
 
+// Eq. rans Enc on the symbols of `row` (four per word) from the last one back, so that decoding runs forward.  The entries
+// do not depend on the state: a word's are fetched while the word after it is coded.
+template <int STRIDE>
+__device__ __forceinline__ void rans_encode_row(const uint4* enc, const uint32_t* row, int words, uint32_t& x, uint32_t& dst) {
+    uint4 nxt[4];
+    uint32_t m4 = row[words - 1];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) nxt[b] = enc[(m4 >> (8 * b)) & 0xffu];
+    m4 = row[max(words - 2, 0)];
+#pragma unroll 1
+    for (int jw = words - 1; jw >= 0; --jw) {
+        uint4 cur[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) { cur[b] = nxt[b]; nxt[b] = enc[(m4 >> (8 * b)) & 0xffu]; }
+        m4 = row[max(jw - 2, 0)];
+#pragma unroll
+        for (int b = 3; b >= 0; --b) rans_step<STRIDE>(x, dst, cur[b]);
+    }
+}
+
 struct StreamQuantised {
     uint32_t hdr0;      // s fp16 | o fp16 << 16
     uint32_t flags;     // 1: all-central fallback, 2: constant stream, 4: refit rejected

@@ -113,15 +113,7 @@ dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_con
         uint32_t xs = 1u << (T.sigma - 9);
         const uint32_t dst0 = dqdev::smem_addr(s_bytesT) + lane;
         uint32_t dst = dst0;   // at most one byte per symbol: 128 rows of kB32 bytes suffice
-#pragma unroll 1
-        for (int jw = (PAIR ? kN / 2 : kN) / 4 - 1; jw >= 0; --jw) {
-            const uint32_t m4 = s_sym[lane * kB32SymWords + jw];
-            uint4 en[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) en[b] = T.enc[(m4 >> (8 * b)) & 0xffu];
-#pragma unroll
-            for (int b = 3; b >= 0; --b) rans_step<kB32>(xs, dst, en[b]);
-        }
+        rans_encode_row<kB32>(T.enc, s_sym + lane * kB32SymWords, (PAIR ? kN / 2 : kN) / 4, xs, dst);
         const uint32_t k = (dst - dst0) / kB32;
         s_xs[lane] = xs;
         s_k[lane] = k;

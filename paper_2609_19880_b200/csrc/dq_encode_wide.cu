@@ -521,15 +521,7 @@ dq_encode_wide_kernel(const __grid_constant__ DqDevTable TD, const __grid_consta
         const uint32_t dst0 = dqdev::smem_addr(s_bytesT) + lane;
         uint32_t dst = dst0;   // the budget test keeps the bytes of a stream below rec - 8
         const uint32_t* row = s_sym + lane * sym_words;
-#pragma unroll 1
-        for (int jw = hs * (PAIR ? kN / 8 : kN / 4) - 1; jw >= 0; --jw) {
-            const uint32_t m4 = row[jw];
-            uint4 en[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) en[b] = T.enc[(m4 >> (8 * b)) & 0xffu];
-#pragma unroll
-            for (int b = 3; b >= 0; --b) rans_step<kWB>(xs, dst, en[b]);
-        }
+        rans_encode_row<kWB>(T.enc, row, hs * (PAIR ? kN / 8 : kN / 4), xs, dst);
         const uint32_t k = (dst - dst0) / kWB;
         s_xs[lane] = xs;
         s_k[lane] = k;
