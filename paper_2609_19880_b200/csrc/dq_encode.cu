@@ -27,23 +27,56 @@ __device__ __forceinline__ void means_of_run(const uint16_t* __restrict__ k, int
         cnt += 32;
     }
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    constexpr int kAheadLoads = 8;   // independent loads in flight; the additions keep token order
-    for (int tb = t0; tb < t0 + cnt; tb += kAheadLoads) {
-        uint2 raw[kAheadLoads];
+    // Independent loads in flight (a window of 128 tokens in four waits, with the rotary tables in sixteen); the
+    // additions keep token order.
+    if (!rope_style) {
+        constexpr int kAhead = 32;
+        for (int tb = t0; tb < t0 + cnt; tb += kAhead) {
+            uint2 raw[kAhead];
 #pragma unroll
-        for (int u = 0; u < kAheadLoads; ++u) {
-            const int tt = min(tb + u, t0 + cnt - 1);
-            raw[u] = *reinterpret_cast<const uint2*>(k + ((size_t)tt * Hkv + h) * kN + 4 * lane);
+            for (int u = 0; u < kAhead; ++u)
+                raw[u] = *reinterpret_cast<const uint2*>(k + ((size_t)min(tb + u, t0 + cnt - 1) * Hkv + h) * kN + 4 * lane);
+            const int n = t0 + cnt - tb;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+                if (u < n) {
+                    float kt[4];
+                    unpack_bf16x4(raw[u], kt);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[e] = __fadd_rn(acc[e], kt[e]);
+                }
         }
+    } else {
+        constexpr int kAhead = 8;
+        const int per = rope_style == DQ_ROPE_HALF ? 4 * (lane & 15) : 2 * lane;   // this lane's place in a position's 64 angles
+        for (int tb = t0; tb < t0 + cnt; tb += kAhead) {
+            uint2 raw[kAhead];
+            float4 cs[kAhead], sn[kAhead];
 #pragma unroll
-        for (int u = 0; u < kAheadLoads; ++u) {
-            if (tb + u >= t0 + cnt) break;
-            float kt[4] = {bf16_bits_to_float(raw[u].x & 0xffffu), bf16_bits_to_float(raw[u].x >> 16),
-                           bf16_bits_to_float(raw[u].y & 0xffffu), bf16_bits_to_float(raw[u].y >> 16)};
-            if (rope_style)
-                warp_rope128(kt, lane, rope_cos + (size_t)pos[tb + u] * 64, rope_sin + (size_t)pos[tb + u] * 64, rope_style);
+            for (int u = 0; u < kAhead; ++u) {
+                const int tt = min(tb + u, t0 + cnt - 1);
+                raw[u] = *reinterpret_cast<const uint2*>(k + ((size_t)tt * Hkv + h) * kN + 4 * lane);
+                const float* c = rope_cos + (size_t)pos[tt] * 64 + per;
+                const float* n = rope_sin + (size_t)pos[tt] * 64 + per;
+                if (rope_style == DQ_ROPE_HALF) {
+                    cs[u] = *reinterpret_cast<const float4*>(c);
+                    sn[u] = *reinterpret_cast<const float4*>(n);
+                } else {
+                    const float2 c2 = *reinterpret_cast<const float2*>(c), n2 = *reinterpret_cast<const float2*>(n);
+                    cs[u] = make_float4(c2.x, c2.y, 0.f, 0.f);
+                    sn[u] = make_float4(n2.x, n2.y, 0.f, 0.f);
+                }
+            }
+            const int n = t0 + cnt - tb;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[e] = __fadd_rn(acc[e], kt[e]);
+            for (int u = 0; u < kAhead; ++u)
+                if (u < n) {
+                    float kt[4];
+                    unpack_bf16x4(raw[u], kt);
+                    warp_rope128(kt, lane, cs[u], sn[u], rope_style);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[e] = __fadd_rn(acc[e], kt[e]);
+                }
         }
     }
     const int t = t0 + cnt;
@@ -80,7 +113,9 @@ dq_means_compute_kernel(const uint16_t* __restrict__ k, int T, int Hkv, int rota
     __shared__ int s_first[kMeansTokens];
     __shared__ int s_n;
     const int lane = threadIdx.x & 31;
+    dqdev::pdl_launch_dependents();
     if (threadIdx.x == 0) s_n = 0;
+    dqdev::pdl_wait_prior_grid();
     __syncthreads();
     {
         const long long tt = (long long)blockIdx.x * kMeansTokens + threadIdx.x;
@@ -242,9 +277,8 @@ cudaError_t dq_launch_means(const DqDevTable& tk, const void* k_bf16, int T, int
     if (T == 0 || Hkv == 0) return cudaSuccess;
     if (mode != DQ_MEAN_COMPUTE) return cudaSuccess;  // carry-forward is done by the encoder warps
     const unsigned blocks = (unsigned)((T + kMeansTokens - 1) / kMeansTokens);
-    dq_means_compute_kernel<<<blocks, 256, 0, st>>>((const uint16_t*)k_bf16, T, Hkv, tk.rotate, seq_id, pos,
-                                                    mean_q, mean_scale, max_windows, rope_cos, rope_sin, rope_style);
-    return cudaGetLastError();
+    return dq_launch_pdl(dq_means_compute_kernel, dim3(blocks), dim3(256), 0, st, (const uint16_t*)k_bf16, T, Hkv, tk.rotate, seq_id, pos,
+                         mean_q, mean_scale, max_windows, rope_cos, rope_sin, rope_style);
 }
 
 // Smallest number of streams for which a call goes to the batch kernels (32 streams per CTA); the
@@ -265,8 +299,11 @@ cudaError_t dq_launch_encode(const DqDevTable& tk, const DqDevTable& tv, const D
     const unsigned blocks = (unsigned)((warps + kEncWarps - 1) / kEncWarps);
     const bool pair = tk.pair != 0;   // the caller has checked that both tables agree
     const dim3 kinds(1, (a.do_k && a.do_v) ? 2 : 1);
-    if (!a.step_flags && warps >= batch_min_streams(4LL * 148 * kDqEncodeBatchStreams * 4))   // enough streams to fill the GPU several times
-        return dq_launch_encode_batch(tk, tv, pk, pv, a, st);
+    // One warp per stream while the call's streams are resident at once (two CTAs of eight warps per SM); beyond that
+    // the batch kernel, whose coding pass is shared.  The option's batches are CTAs of 32 streams.
+    const long long batch_min = batch_min_streams(-1);
+    if (!a.step_flags && (batch_min < 0 ? warps * kinds.y > 2LL * 148 * kEncWarps : warps >= batch_min))
+        return dq_launch_encode_batch(tk, tv, pk, pv, a, batch_min < 0 ? 0 : kDqEncodeBatchStreams, st);
     if (a.step_flags) {   // decode step: big CTAs, so that few SMs are kept from the attention kernel
         constexpr int kStepWarps = DQ_STEP_ENC_WARPS;
         return dq_launch_pdl(pair ? dq_encode_kernel<1, kStepWarps, true> : dq_encode_kernel<1, kStepWarps, false>,

@@ -23,11 +23,9 @@ using dqdrift::WarpGroup;
 // Rotary position embedding of a head vector held 4 values per lane (element 4 lane + e), in
 // binary32 with every product and sum rounded once.  DQ_ROPE_HALF pairs element j with j + 64
 // (the partner sits in lane ^ 16), DQ_ROPE_PAIRS pairs 2j with 2j + 1 (same lane).
-// cs / sn: this position's 64 cosines / sines.
-__device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, const float* cs, const float* sn, int style) {
+// c / s: this lane's cosines / sines, of angles 4 (lane & 15) .. + 3 (halves) or 2 lane, 2 lane + 1 (pairs).
+__device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, float4 c, float4 s, int style) {
     if (style == DQ_ROPE_HALF) {
-        const float4 c = *reinterpret_cast<const float4*>(cs + 4 * (lane & 15));
-        const float4 s = *reinterpret_cast<const float4*>(sn + 4 * (lane & 15));
         const float cc[4] = {c.x, c.y, c.z, c.w}, ss[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -37,8 +35,6 @@ __device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, const floa
             v[e] = (lane < 16) ? __fsub_rn(mine, cross) : __fadd_rn(mine, cross);
         }
     } else {
-        const float2 c = *reinterpret_cast<const float2*>(cs + 2 * lane);
-        const float2 s = *reinterpret_cast<const float2*>(sn + 2 * lane);
         const float a0 = v[0], b0 = v[1], a1 = v[2], b1 = v[3];
         v[0] = __fsub_rn(__fmul_rn(a0, c.x), __fmul_rn(b0, s.x));
         v[1] = __fadd_rn(__fmul_rn(b0, c.x), __fmul_rn(a0, s.x));
@@ -46,8 +42,19 @@ __device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, const floa
         v[3] = __fadd_rn(__fmul_rn(b1, c.y), __fmul_rn(a1, s.y));
     }
 }
-
-// ------------------------------------------------------------------------ drift
+// The same with cs / sn: this position's 64 cosines / sines.
+__device__ __forceinline__ void warp_rope128(float (&v)[4], int lane, const float* cs, const float* sn, int style) {
+    float4 c, s;
+    if (style == DQ_ROPE_HALF) {
+        c = *reinterpret_cast<const float4*>(cs + 4 * (lane & 15));
+        s = *reinterpret_cast<const float4*>(sn + 4 * (lane & 15));
+    } else {
+        const float2 c2 = *reinterpret_cast<const float2*>(cs + 2 * lane), s2 = *reinterpret_cast<const float2*>(sn + 2 * lane);
+        c = make_float4(c2.x, c2.y, 0.f, 0.f);
+        s = make_float4(s2.x, s2.y, 0.f, 0.f);
+    }
+    warp_rope128(v, lane, c, s, style);
+}
 
 // Table of one tensor kind into shared memory, by all threads of the CTA (at least 32).
 __device__ __forceinline__ void load_enc_table(EncTable& T, const DqDevTable& TK, const DqDevTable& TV,
@@ -452,10 +459,11 @@ __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, co
 
 }  // namespace dqenc
 
-// Batch kernels (dq_encode_batch.cu): streams per CTA, and the launch of one tensor kind or both.
+// Batch kernels (dq_encode_batch.cu): most streams per CTA, and the launch of one tensor kind or both; per: streams per
+// CTA, 0: by the size of the call.
 constexpr int kDqEncodeBatchStreams = 32;
 cudaError_t dq_launch_encode_batch(const DqDevTable& tk, const DqDevTable& tv, const DqPairEnc& pk, const DqPairEnc& pv,
-                                   const DqEncodeArgs& a, cudaStream_t st);
+                                   const DqEncodeArgs& a, int per, cudaStream_t st);
 // Token-wide streams (dq_encode_wide.cu); per: streams per CTA, 0: by the size of the call.
 cudaError_t dq_launch_encode_wide(const DqDevTable& tk, const DqDevTable& tv, const DqPairEnc& pk, const DqPairEnc& pv,
                                   const DqEncodeArgs& a, int per, cudaStream_t st);

@@ -30,7 +30,7 @@ constexpr int batch_min_blocks(int M, bool pair) { return pair || M > 9 ? 4 : M 
 // second kind's launch (`second`) does not wait for the first's, it only ends after it.
 template <int M, bool PAIR>
 __global__ void __launch_bounds__(kB32Warps * 32, batch_min_blocks(M, PAIR))
-dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_constant__ DqPairEnc PD, const DqEncodeArgs a, bool is_v,
+dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_constant__ DqPairEnc PD, const DqEncodeArgs a, int per, bool is_v,
                          bool second) {
     __shared__ __align__(16) EncTable T;
     __shared__ uint32_t s_sym[kB32 * kB32SymWords];
@@ -47,8 +47,8 @@ dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_con
     dqdev::pdl_launch_dependents();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long total = (long long)a.T * a.Hkv;
-    const long long first = (long long)blockIdx.x * kB32;
-    const int ns = (int)min((long long)kB32, total - first);
+    const long long first = (long long)blockIdx.x * per;
+    const int ns = (int)min((long long)per, total - first);
     const int rec = TD.rec;
     const bool has_mean = TD.has_mean, rope = !is_v && a.rope_style;
 
@@ -133,7 +133,7 @@ dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_con
     if (second) dqdev::pdl_wait_prior_grid();   // the first kind's kernel: whoever waits for this one may read both
 }
 
-using BatchKernel = void (*)(DqDevTable, DqPairEnc, DqEncodeArgs, bool, bool);
+using BatchKernel = void (*)(DqDevTable, DqPairEnc, DqEncodeArgs, int, bool, bool);
 
 template <bool PAIR>
 BatchKernel kernel_for(int M) {
@@ -156,17 +156,25 @@ BatchKernel kernel_for(int M) {
 
 }  // namespace
 
+// Streams per CTA (per = 0): 32 once that fills the GPU about three times, fewer below, so that every SM gets its eight
+// CTAs: the coding pass costs a CTA the same for 4 and for 32 streams.
 cudaError_t dq_launch_encode_batch(const DqDevTable& tk, const DqDevTable& tv, const DqPairEnc& pk, const DqPairEnc& pv,
-                                   const DqEncodeArgs& a, cudaStream_t st) {
+                                   const DqEncodeArgs& a, int per, cudaStream_t st) {
     const long long streams = (long long)a.T * a.Hkv;
-    const dim3 grid((unsigned)((streams + kB32 - 1) / kB32)), block(kB32Warps * 32);
+    if (per <= 0) {
+        const long long resident = 148LL * DQ_B32_MINB / ((a.do_k && a.do_v) ? 2 : 1);
+        per = (int)((streams + resident - 1) / resident);
+        per = (per + kB32Warps - 1) / kB32Warps * kB32Warps;   // whole rounds of the CTA's warps
+    }
+    per = per > kB32 ? kB32 : per;
+    const dim3 grid((unsigned)((streams + per - 1) / per)), block(kB32Warps * 32);
     bool second = false;
     for (int kind = 0; kind < 2; ++kind) {
         if (kind == 0 ? !a.do_k : !a.do_v) continue;
         const DqDevTable& t = kind == 0 ? tk : tv;
         const auto kernel = t.pair ? kernel_for<true>(t.M) : kernel_for<false>(t.M);
         if (!kernel) return cudaErrorInvalidValue;
-        const cudaError_t e = dq_launch_pdl(kernel, grid, block, 0, st, t, kind == 0 ? pk : pv, a, kind == 1, second);
+        const cudaError_t e = dq_launch_pdl(kernel, grid, block, 0, st, t, kind == 0 ? pk : pv, a, per, kind == 1, second);
         if (e != cudaSuccess) return e;
         second = true;
     }
