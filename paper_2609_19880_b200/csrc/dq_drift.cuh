@@ -41,6 +41,7 @@ struct EncTable {
     int M, rec, mstar, budget_bits, has_mean, rotate;
     int early_exit, sigma;         // codec variants: Drift tries its end multiplier first; bits of final state (32 / 24)
     int pair;                      // paired symbols
+    float pair_dr;                 // DqDevTable::pair_dr
     int fast;                      // DqDevTable::drift_fast
     uint32_t central;              // the all-central stream's four levels of a lane, one per byte
 };

@@ -85,6 +85,7 @@ __device__ __forceinline__ void load_enc_table(EncTable& T, const DqDevTable& TK
         T.has_mean = is_v ? TV.has_mean : TK.has_mean; T.rotate = is_v ? TV.rotate : TK.rotate;
         T.early_exit = is_v ? TV.early_exit : TK.early_exit; T.sigma = sigma;
         T.pair = pair;
+        T.pair_dr = is_v ? TV.pair_dr : TK.pair_dr;
         const uint32_t ms = (uint32_t)T.mstar, us = (uint32_t)(is_v ? TV.ustar : TK.ustar), M = (uint32_t)T.M;
         T.central = pair ? (us / M) * 0x00010001u + (us % M) * 0x01000100u : ms * 0x01010101u;
     }
@@ -177,9 +178,63 @@ __device__ __forceinline__ uint32_t drift(const EncTable& T, const float (&z)[4]
 // Drift for the paired-symbol variant: a lane's values (0, 1) and (2, 3) are two rANS symbols; each takes
 // the pair u = a M + b that minimises (D_a + D_b) + lambda r_u, the lowest u among equal costs (rows a in
 // ascending order, each reduced pairwise with the left operand winning ties, a later row replacing the best
-// only when strictly cheaper: the same winner as an ascending scan with a strict comparison).  Bracket: hi = 16 (max D - min D), D over single values as above.
+// only when strictly cheaper: the same winner as an ascending scan with a strict comparison).  Bracket:
+// hi = 16 (max D - min D), D over single values as above.
+// One sweep: the two winners' keys (ceil(65536 r_u) << 8 | u) and the code length.
 template <int M>
-__device__ __forceinline__ uint32_t drift_pair(const EncTable& T, const float (&z)[4], float s, float o, uint32_t& sym_packed) {
+__device__ __forceinline__ uint32_t pair_sweep(const EncTable& T, const float (&D)[4][M], float lam, uint32_t (&win)[2]) {
+    uint32_t cost_sum = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        float rc[M];
+        uint32_t rkey[M];
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+            float c[M];
+            uint32_t key[M];
+#pragma unroll
+            for (int b = 0; b < M; ++b) {
+                const uint2 e = T.prk[a * M + b];
+                c[b] = __fmaf_rn(lam, __uint_as_float(e.x), __fadd_rn(D[2 * p][a], D[2 * p + 1][b]));
+                key[b] = e.y;
+            }
+#pragma unroll
+            for (int w = 1; w < M; w <<= 1)
+#pragma unroll
+                for (int b = 0; b + w < M; b += 2 * w)
+                    if (c[b + w] < c[b]) { c[b] = c[b + w]; key[b] = key[b + w]; }
+            rc[a] = c[0];
+            rkey[a] = key[0];
+        }
+#pragma unroll
+        for (int w = 1; w < M; w <<= 1)   // row winners, the left (lower a) operand wins ties
+#pragma unroll
+            for (int a = 0; a + w < M; a += 2 * w)
+                if (rc[a + w] < rc[a]) { rc[a] = rc[a + w]; rkey[a] = rkey[a + w]; }
+        win[p] = rkey[0];
+        cost_sum += rkey[0];
+    }
+    return __reduce_add_sync(kFull, cost_sum >> 8);   // two pair indices (< 81 each) stay below bit 8
+}
+
+// Cost of pair u at lambda = 0 for the values (za, zb), approximately.
+template <int M>
+__device__ __forceinline__ float pair_distance(float za, float zb, float s, float o, uint32_t u) {
+    const float da = za - fmaf((float)(u / M), s, o), db = zb - fmaf((float)(u % M), s, o);
+    return fmaf(da, da, db * db);
+}
+
+// The bisection's outcome in about five sweeps instead of 13.  A pair's winner moves to ever cheaper pairs as lambda
+// grows, so the code length falls with lambda and the bisection ends in the cell (J, J + 1] of its 4096-point grid
+// between the last length over the budget and the first within it -- whatever the order in which points are looked
+// at.  Two sweeps bracket J around its usual place; between the bracket's ends few pairs change their winner, each
+// at a lambda that its two winners give in closed form, and the order statistic of those is J; sweeps at the exact
+// lambda_{J+1} and lambda_J (the chain of square roots replayed) confirm it or move the bracket.
+// Rounding could make a length rise with lambda only between points closer than 2^-21 of the largest cost over the
+// smallest difference of two r: the search is left (the bisection runs) where neighbouring grid points are.
+template <int M>
+static __device__ __noinline__ uint2 drift_pair_search(const EncTable& T, float z0, float z1, float z2, float z3, float s, float o) {
+    const float z[4] = {z0, z1, z2, z3};
     float D[4][M];
     float maxD = -INFINITY, minD = INFINITY;
 #pragma unroll
@@ -193,62 +248,140 @@ __device__ __forceinline__ uint32_t drift_pair(const EncTable& T, const float (&
             minD = fminf(minD, D[e][m]);
         }
     }
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        maxD = fmaxf(maxD, __shfl_xor_sync(kFull, maxD, d));
-        minD = fminf(minD, __shfl_xor_sync(kFull, minD, d));
-    }
+    maxD = dqdev::warp_max(maxD);
+    minD = dqdev::warp_min(minD);
     const uint32_t budget = (uint32_t)T.budget_bits << 16;
-    float lam_hi = __fmul_rn(16.0f, __fsub_rn(maxD, minD));
-    float lam_lo = __fmul_rn(lam_hi, 0x1p-40f);
-    uint32_t len = 0, psym[2] = {0u, 0u};
+    const float hi0 = __fmul_rn(16.0f, __fsub_rn(maxD, minD)), lo0 = __fmul_rn(hi0, 0x1p-40f);
+    constexpr float kG = 102.4f;
+    uint32_t win[2] = {0u, 0u};
+
+    if (hi0 > 0x1p-38f && hi0 < 0x1p80f && T.pair_dr > 0.f) {
+        const float lg_hi = dqdrift::lg2_approx(hi0);
+        int jl = 0, jh = 4096, j = 4096 + (int)(kG * (dqdrift::lg2_approx(0.25f * s * s) - lg_hi)), step = 48, J = 0;
+        j = min(max(j, 200), 4000);
+        bool have_l = false, have_h = false;
+        uint32_t kl[2] = {0u, 0u}, kh[2] = {0u, 0u}, kf[2] = {0u, 0u}, len_h = 0;
+        float lam = hi0 * dqdrift::exp2_approx((float)(j - 4096) * (1.f / kG)), lam_lo = 0.f;
+        int phase = 0;   // 0: bracket, 1: lambda_{J+1}, 2: lambda_J
+#pragma unroll 1
+        for (int it = 0; it < 11; ++it) {
+            const uint32_t len = pair_sweep<M>(T, D, lam, win);
+            const bool over = len > budget;
+            if (phase == 2 && over) {   // confirmed: the winners at lambda_{J+1}
+                const float far = maxD + maxD + lam * 8.f;   // no cost of a winner is larger
+                if (lam * (0.0067f * T.pair_dr) < 0x1p-21f * far) break;
+                const uint32_t u0 = kf[0] & 0xffu, u1 = kf[1] & 0xffu;
+                return make_uint2(0u, (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24));
+            }
+            const int at = phase == 0 ? j : phase == 1 ? J + 1 : J;
+            if (over) { jl = at; kl[0] = win[0]; kl[1] = win[1]; have_l = true; }
+            else { jh = at; kh[0] = win[0]; kh[1] = win[1]; len_h = len; have_h = true; }
+            if (phase == 1 && !over) {
+                kf[0] = win[0]; kf[1] = win[1];
+                phase = 2;
+                lam = lam_lo;
+                continue;
+            }
+            if (!have_l || !have_h) {
+                j += over ? step : -step;
+                step *= 3;
+                if (j < 2 || j > 4090) break;
+                lam = hi0 * dqdrift::exp2_approx((float)(j - 4096) * (1.f / kG));
+                continue;
+            }
+            // lambdas at which the pairs leave their winner at jl for the one at jh, and what that saves
+            float t[2];
+            uint32_t w[2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const uint32_t ul = kl[p] & 0xffu, uh = kh[p] & 0xffu;
+                const float dr = __uint_as_float(T.prk[ul].x) - __uint_as_float(T.prk[uh].x);
+                const float dD = pair_distance<M>(z[2 * p], z[2 * p + 1], s, o, uh) - pair_distance<M>(z[2 * p], z[2 * p + 1], s, o, ul);
+                w[p] = (kl[p] >> 8) - (kh[p] >> 8);
+                t[p] = (ul != uh && dr > 0.f) ? fmaxf(dD * dqdrift::rcp_approx(dr), 0.f) : 0.f;
+            }
+            float tc = INFINITY;
+            int k = 0;
+#pragma unroll 1
+            for (; k < 40; ++k) {   // largest first, until the length exceeds the budget again
+                float m = 0.f;
+                dqdrift::max_if_less(m, t[0], tc);
+                dqdrift::max_if_less(m, t[1], tc);
+                tc = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(m)));
+                if (!(tc > 0.f)) break;
+                uint32_t sum = 0;
+                dqdrift::add_if_not_less(sum, t[0], tc, w[0]);
+                dqdrift::add_if_not_less(sum, t[1], tc, w[1]);
+                if (len_h + __reduce_add_sync(kFull, sum) > budget) break;
+            }
+            if (k == 40 || !(tc > 0.f)) break;
+            J = 4096 + (int)floorf(kG * (dqdrift::lg2_approx(tc) - lg_hi));
+            J = min(max(J, jl), jh - 1);
+            if (J < 1 || J > 4094) break;
+            float lo = lo0, hi = hi0;
+#pragma unroll 1
+            for (int b = 11; b >= 0; --b) {
+                const float mid = __fsqrt_rn(__fmul_rn(lo, hi));
+                if ((J >> b) & 1) lo = mid; else hi = mid;
+            }
+            lam_lo = lo;
+            lam = hi;
+            phase = 1;
+        }
+    }
+
+    float lam_hi = hi0, lam_lo = lo0;
+    uint32_t len = 0;
     float lam_e = lam_hi;
     if (T.early_exit)
         for (int i = 0; i < 12; ++i) lam_e = __fsqrt_rn(__fmul_rn(lam_lo, lam_e));
 #pragma unroll 1
     for (int it = T.early_exit ? -1 : 0; it <= 12; ++it) {
         const float lam = (it < 0) ? lam_e : (it < 12) ? __fsqrt_rn(__fmul_rn(lam_lo, lam_hi)) : lam_hi;
-        uint32_t cost_sum = 0;
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float rc[M];
-            uint32_t rkey[M];
-#pragma unroll
-            for (int a = 0; a < M; ++a) {
-                float c[M];
-                uint32_t key[M];
-#pragma unroll
-                for (int b = 0; b < M; ++b) {
-                    const uint2 e = T.prk[a * M + b];
-                    c[b] = __fmaf_rn(lam, __uint_as_float(e.x), __fadd_rn(D[2 * p][a], D[2 * p + 1][b]));
-                    key[b] = e.y;
-                }
-#pragma unroll
-                for (int w = 1; w < M; w <<= 1)
-#pragma unroll
-                    for (int b = 0; b + w < M; b += 2 * w)
-                        if (c[b + w] < c[b]) { c[b] = c[b + w]; key[b] = key[b + w]; }
-                rc[a] = c[0];
-                rkey[a] = key[0];
-            }
-#pragma unroll
-            for (int w = 1; w < M; w <<= 1)   // row winners, the left (lower a) operand wins ties
-#pragma unroll
-                for (int a = 0; a + w < M; a += 2 * w)
-                    if (rc[a + w] < rc[a]) { rc[a] = rc[a + w]; rkey[a] = rkey[a + w]; }
-            psym[p] = rkey[0];
-            cost_sum += rkey[0];
-        }
-        len = __reduce_add_sync(kFull, cost_sum >> 8);   // two pair indices (< 81 each) stay below bit 8
+        len = pair_sweep<M>(T, D, lam, win);
         if (it < 0) {
             if (len <= budget) break;
         } else if (it < 12) {
             if (len <= budget) lam_hi = lam; else lam_lo = lam;
         }
     }
-    const uint32_t u0 = psym[0] & 0xffu, u1 = psym[1] & 0xffu;
-    sym_packed = (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24);
-    return len;
+    const uint32_t u0 = win[0] & 0xffu, u1 = win[1] & 0xffu;
+    return make_uint2(len, (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24));
+}
+
+// Levels of the nearest pairs when they fit the budget (every test of the bisection then passes and lambda ends too
+// small to move any pair) and no value is within rounding of a midpoint.
+template <int M>
+__device__ __forceinline__ bool drift_pair_nearest(const EncTable& T, const float (&z)[4], float s, float o, float zmin, float zmax,
+                                                   uint32_t& sym) {
+    if (!(s > 0x1p-30f && s < 0x1p40f)) return false;
+    const float inv = dqdrift::rcp_approx(s), shift = -o * inv;
+    const float vmax = fmaf(zmax, inv, shift), vmin = fmaf(zmin, inv, shift);
+    const float reach = fmaxf(vmax, (float)(M - 1) - vmin);
+    const float mag = fmaxf(fmaxf(fabsf(zmin), fabsf(zmax)), fmaxf(fabsf(o), fabsf(o + (float)(M - 1) * s))) * inv;
+    if (!(mag < 1024.f && reach < 64.f)) return false;
+    const float E = 1.5f * 0x1p-24f * (2.f * mag + 4.f * reach + (float)M + 2.f * reach * reach);
+    float near[4], mid = 1.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float v = fmaf(z[e], inv, shift);
+        near[e] = fminf(fmaxf((v + 12582912.f) - 12582912.f, 0.f), (float)(M - 1));
+        mid = fminf(mid, fabsf(fabsf(v - near[e]) - 0.5f));
+    }
+    const uint32_t u0 = (uint32_t)(int)fmaf(near[0], (float)M, near[1]), u1 = (uint32_t)(int)fmaf(near[2], (float)M, near[3]);
+    const uint32_t len = __reduce_add_sync(kFull, (T.prk[u0].y >> 8) + (T.prk[u1].y >> 8));
+    sym = (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24);
+    return len <= ((uint32_t)T.budget_bits << 16) && __all_sync(kFull, mid > E);
+}
+
+// Length of the assignment (0: known to be within the budget); sym: its levels, one per byte.
+template <int M>
+__device__ __forceinline__ uint32_t drift_pair(const EncTable& T, const float (&z)[4], float s, float o, float zmin, float zmax,
+                                               uint32_t& sym) {
+    if (drift_pair_nearest<M>(T, z, s, o, zmin, zmax, sym)) return 0u;
+    const uint2 r = drift_pair_search<M>(T, z[0], z[1], z[2], z[3], s, o);
+    sym = r.y;
+    return r.x;
 }
 
 // ---------------------------------------------------------------------- encoder
@@ -437,7 +570,7 @@ __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, co
     const float o = mn;                                             // FitMinMax, Eq. (affine_token)
     const float s = __fdiv_rn(__fsub_rn(mx, mn), (float)(M - 1));
     uint32_t sym = 0u;
-    if (PAIR) drift_pair<M>(T, z, s, o, sym); else drift<M>(T, z, s, o, mn, mx, sym);
+    if (PAIR) drift_pair<M>(T, z, s, o, mn, mx, sym); else drift<M>(T, z, s, o, mn, mx, sym);
     uint32_t hdr;                                                   // Refit, fp16 metadata
     const RefitScale sc = refit_scale(fmaxf(fabsf(mn), fabsf(mx)));
     const RefitSums h = refit_sums(z, sc, sym);
@@ -451,7 +584,7 @@ __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, co
         r.flags = 4u;
     }
     if (!(sf > 0.0f)) { r.flags |= 2u; return r; }
-    const uint32_t len = PAIR ? drift_pair<M>(T, z, sf, of, sym) : drift<M>(T, z, sf, of, mn, mx, sym);   // second Drift, fp16 grid
+    const uint32_t len = PAIR ? drift_pair<M>(T, z, sf, of, mn, mx, sym) : drift<M>(T, z, sf, of, mn, mx, sym);   // second Drift, fp16 grid
     r.hdr0 = hdr;
     if (len > ((uint32_t)T.budget_bits << 16)) r.flags |= 1u; else r.sym = sym;
     return r;

@@ -298,6 +298,11 @@ int dq_host_build(int levels, double bits_per_elem, const dq_table_opts* opts, d
             out->penc.R[u] = t.pair_R[u];
             c += (uint32_t)t.pair_f[u];
         }
+        std::vector<float> costs(out->penc.r, out->penc.r + levels * levels);
+        std::sort(costs.begin(), costs.end());
+        d.pair_dr = 0.f;
+        for (size_t i = 1; i < costs.size(); ++i)
+            if (costs[i] > costs[i - 1] && (d.pair_dr == 0.f || costs[i] - costs[i - 1] < d.pair_dr)) d.pair_dr = costs[i] - costs[i - 1];
     }
     std::memcpy(d.lut, t.lut, sizeof d.lut);
     return DQ_OK;
