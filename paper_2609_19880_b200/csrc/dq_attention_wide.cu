@@ -306,8 +306,10 @@ __device__ __forceinline__ void wide_pass(Chain& ck, Chain& cv, uint32_t ringk, 
             ldmatrix_x4_trans(a1, vtile + ld_off + 16 * 32);
             mma_f16_16816(o, a0, pb_hi[0][0], pb_hi[0][1]);
             mma_f16_16816(o, a1, pb_hi[1][0], pb_hi[1][1]);
-            mma_f16_16816(o, a0, pb_lo[0][0], pb_lo[0][1]);
-            mma_f16_16816(o, a1, pb_lo[1][0], pb_lo[1][1]);
+            float ol[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_f16_16816(ol, a0, pb_lo[0][0], pb_lo[0][1]);
+            mma_f16_16816(ol, a1, pb_lo[1][0], pb_lo[1][1]);
+            o[0] += ol[0]; o[1] += ol[1]; o[2] += ol[2]; o[3] += ol[3];
             const uint32_t oa = o_addr + cg * 64;
             if (2 * (lane & 3) < G) { sts32f(oa, o[0]); sts32f(oa + 32, o[2]); }
             if (2 * (lane & 3) + 1 < G) { sts32f(oa + kORow * 4, o[1]); sts32f(oa + kORow * 4 + 32, o[3]); }

@@ -143,7 +143,7 @@ constexpr int kEncWarps = 8;
 template <int M, bool PAIR>
 __device__ __noinline__ StreamQuantised quantise_m(const EncTable& T, float z0, float z1, float z2, float z3) {
     const float z[4] = {z0, z1, z2, z3};
-    return quantise_values<M, PAIR>(T, z);
+    return quantise_values<M, PAIR, true>(T, z);
 }
 template <bool PAIR>
 __device__ __forceinline__ StreamQuantised quantise_any(const EncTable& T, const float (&z)[4]) {
@@ -225,6 +225,7 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
     split_stream(a, wid, t, h);
     const int Hkv = a.Hkv;
     if (tok_pos(a, t) < 0) return;   // decode-step mode: an empty sequence has no new token
+    const int sl = a.slot[t];        // needed at the end, on its way meanwhile
     uint8_t* cont = is_v ? a.v_cont : a.k_cont;
 
     const StreamQuantised sq = quantise_stream<PAIR>(T, a, is_v, t, h, lane);
@@ -247,7 +248,6 @@ dq_encode_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ 
     __syncwarp();
     asm volatile("" ::: "memory");
     const uint32_t hdr0 = sq.hdr0;
-    const int sl = a.slot[t];
     uint8_t* rec = cont + (((size_t)(sl / DQ_PAGE_TOKENS) * Hkv + h) * DQ_PAGE_TOKENS +
                            (size_t)(sl % DQ_PAGE_TOKENS)) * T.rec;
     const int pay = 4 + (T.sigma >> 3);              // first payload byte: after (s, o) and the final state

@@ -558,7 +558,9 @@ static __device__ __noinline__ uint32_t refit_binary64(float z0, float z1, float
 // Steps 2-6 of Algorithm 1 by one warp on the rotated, mean-free values of a stream: min-max grid, drift, refit,
 // fp16 metadata, second drift.  M: the table's levels.
 // PAIR: its rANS symbols are pairs of levels.
-template <int M, bool PAIR>
+// COMPACT: both Drift calls run the same code in a loop -- for calls of a few streams, whose time is the way through the
+// code once, with the instruction cache cold.
+template <int M, bool PAIR, bool COMPACT>
 __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, const float (&z)[4]) {
     const float mx = dqdev::warp_max(fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])));
     const float mn = dqdev::warp_min(fminf(fminf(z[0], z[1]), fminf(z[2], z[3])));
@@ -567,24 +569,27 @@ __device__ __forceinline__ StreamQuantised quantise_values(const EncTable& T, co
     r.flags = 0u;
     r.hdr0 = (uint32_t)__half_as_ushort(__float2half_rn(mn)) << 16;
     if (!(mx > mn)) { r.flags = 2u; return r; }
-    const float o = mn;                                             // FitMinMax, Eq. (affine_token)
-    const float s = __fdiv_rn(__fsub_rn(mx, mn), (float)(M - 1));
-    uint32_t sym = 0u;
-    if (PAIR) drift_pair<M>(T, z, s, o, mn, mx, sym); else drift<M>(T, z, s, o, mn, mx, sym);
-    uint32_t hdr;                                                   // Refit, fp16 metadata
-    const RefitScale sc = refit_scale(fmaxf(fabsf(mn), fabsf(mx)));
-    const RefitSums h = refit_sums(z, sc, sym);
-    if (!sc.ok || !refit_finish(sc, (float)kN, (float)h.SA, (float)h.SB, (float)h.Sm, (float)(kN * h.Smm - h.Sm * h.Sm), hdr))
-        hdr = refit_binary64(z[0], z[1], z[2], z[3], sym, s, o);
-    float sf = __half2float(__ushort_as_half((unsigned short)(hdr & 0xffffu))), of = __half2float(__ushort_as_half((unsigned short)(hdr >> 16)));
-    if (!(isfinite(sf) && sf > 0.0f && isfinite(of))) {
-        const __half s16 = __float2half_rn(s), o16 = __float2half_rn(o);
-        hdr = (uint32_t)__half_as_ushort(s16) | ((uint32_t)__half_as_ushort(o16) << 16);
-        sf = __half2float(s16); of = __half2float(o16);
-        r.flags = 4u;
+    float s = __fdiv_rn(__fsub_rn(mx, mn), (float)(M - 1)), o = mn; // FitMinMax, Eq. (affine_token)
+    uint32_t sym = 0u, len = 0u, hdr = 0u;
+#pragma unroll (COMPACT ? 1 : 2)
+    for (int pass = 0; pass < 2; ++pass) {
+        len = PAIR ? drift_pair<M>(T, z, s, o, mn, mx, sym) : drift<M>(T, z, s, o, mn, mx, sym);
+        if (pass == 1) break;
+        // Refit, fp16 metadata; the second Drift runs on the fp16 grid
+        const RefitScale sc = refit_scale(fmaxf(fabsf(mn), fabsf(mx)));
+        const RefitSums h = refit_sums(z, sc, sym);
+        if (!sc.ok || !refit_finish(sc, (float)kN, (float)h.SA, (float)h.SB, (float)h.Sm, (float)(kN * h.Smm - h.Sm * h.Sm), hdr))
+            hdr = refit_binary64(z[0], z[1], z[2], z[3], sym, s, o);
+        float sf = __half2float(__ushort_as_half((unsigned short)(hdr & 0xffffu))), of = __half2float(__ushort_as_half((unsigned short)(hdr >> 16)));
+        if (!(isfinite(sf) && sf > 0.0f && isfinite(of))) {
+            const __half s16 = __float2half_rn(s), o16 = __float2half_rn(o);
+            hdr = (uint32_t)__half_as_ushort(s16) | ((uint32_t)__half_as_ushort(o16) << 16);
+            sf = __half2float(s16); of = __half2float(o16);
+            r.flags = 4u;
+        }
+        if (!(sf > 0.0f)) { r.flags |= 2u; return r; }
+        s = sf; o = of;
     }
-    if (!(sf > 0.0f)) { r.flags |= 2u; return r; }
-    const uint32_t len = PAIR ? drift_pair<M>(T, z, sf, of, mn, mx, sym) : drift<M>(T, z, sf, of, mn, mx, sym);   // second Drift, fp16 grid
     r.hdr0 = hdr;
     if (len > ((uint32_t)T.budget_bits << 16)) r.flags |= 1u; else r.sym = sym;
     return r;

@@ -92,7 +92,7 @@ dq_encode_batch32_kernel(const __grid_constant__ DqDevTable TD, const __grid_con
             remove_mean(z, q4, sc);
         }
         load(i + kB32Warps, raw, q4, sc);
-        const StreamQuantised sq = quantise_values<M, PAIR>(T, z);
+        const StreamQuantised sq = quantise_values<M, PAIR, false>(T, z);
         if (PAIR) {   // the lane's two pair indices u = a M + b
             const uint32_t u0 = (sq.sym & 0xffu) * M + ((sq.sym >> 8) & 0xffu), u1 = ((sq.sym >> 16) & 0xffu) * M + (sq.sym >> 24);
             reinterpret_cast<uint16_t*>(s_sym + i * kB32SymWords)[lane] = (uint16_t)(u0 | (u1 << 8));
