@@ -1150,7 +1150,7 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
     const int G1 = a.Hq / a.Hkv, G = G1 * q_len;   // rows per KV head
     const bool wide = tk.hs > 1;   // token-wide streams: main kernel of dq_attention_wide.cu
     Layout L = make_layout(nw, tk.rec, tv.rec, a.B, G);
-    const int small = wide ? 0 : dq_attn_small_pick_warps(tk, tv, a.B, a.Hkv, a.max_pages, sm_count, smem_max);
+    const int small = dq_attn_small_pick_warps(tk, tv, a.B, a.Hkv, a.max_pages, sm_count, smem_max);
     if (small) {
         nw = small;
     } else if (wide) {
