@@ -207,6 +207,7 @@ int dq_decode_attention_multi(const dq_tables* tk, const dq_tables* tv, const vo
     a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.sm_scale = sm_scale;
     a.resid_k = resid_k_bf16; a.resid_v = resid_v_bf16; a.resid_lens = resid_lens; a.resid_cap = resid_cap;
     a.q_len = q_len;
+    a.workspace_bytes = workspace_bytes;
     a.fused = 0;
     const cudaError_t e = dq_launch_attention(tk->dev, tv->dev, a, static_cast<cudaStream_t>(cuda_stream));
     if (e != cudaSuccess) return cuda_fail(e, "decode attention");
@@ -268,6 +269,7 @@ int dq_decode_attention_static(const dq_tables* tk, const dq_tables* tv, const v
     a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.sm_scale = sm_scale;
     a.resid_k = nullptr; a.resid_v = nullptr; a.resid_lens = nullptr; a.resid_cap = 0;
     a.q_len = 1;
+    a.workspace_bytes = 0;
     a.fused = 0;
     e = dq_launch_attention_static(tk->dev, tv->dev, a, static_cast<cudaStream_t>(cuda_stream));
     if (e != cudaSuccess) return cuda_fail(e, "decode attention (static scratch)");

@@ -35,7 +35,7 @@ namespace {
 constexpr int kTileStride = 32;        // bytes per token row of a [32 tok][16 ch] fp16 tile; the
                                        // 16 pad bytes of the K tile rows hold (sK, oK, sV, oV)
 constexpr int kTileBytes = kChunk * kTileStride;
-constexpr int kKTail = 32;             // bytes after a warp's K records: q'.mean of its window, per head
+constexpr int kRowWarps16 = 8;         // warps of the 16-row kernel: output slots of 8 KB leave room for no more
 
 struct Item {
     int b, h, blk, len, bg, valid;
@@ -52,9 +52,10 @@ struct Layout {
 
 __host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
 
-__host__ __device__ inline Layout make_layout(int nw, int rec_k, int rec_v, int B, int G) {
+// rows: query rows of a KV head that the kernel's tiles hold (8 or 16)
+__host__ __device__ inline Layout make_layout(int nw, int rec_k, int rec_v, int B, int G, int rows) {
     Layout L;
-    L.stage_k = align16(kChunk * rec_k) + kKTail;
+    L.stage_k = align16(kChunk * rec_k) + 4 * rows;   // + q'.mean of the warp's window, per row
     L.stage_v = align16(kChunk * rec_v);
     L.warp_tile_bytes = 2 * kTileBytes;             // K tile (+ per-token metadata), V tile
     L.warp_obuf_bytes = G * kORow * 4;              // this warp's O[g][channel], l, off
@@ -63,9 +64,9 @@ __host__ __device__ inline Layout make_layout(int nw, int rec_k, int rec_v, int 
     int o = 0;
     L.off_lutk = o; o += 256 * 32 * 4;
     L.off_lutv = o; o += 256 * 32 * 4;
-    L.off_q16 = o; o += 2 * kQ16Bytes;
-    L.off_qsum = o; o += 2 * DQ_MAX_GROUP * 4;
-    L.off_red = o; o += (kMaxWarps + 2) * DQ_MAX_GROUP * 4;
+    L.off_q16 = o; o += 2 * (rows / 8) * kQ16Bytes;
+    L.off_qsum = o; o += 2 * rows * 4;
+    L.off_red = o; o += (kMaxWarps + 2) * rows * 4;
     L.off_pages = o; o += kMaxWarps * 3 * 2 * 4 + 16;   // per warp: page ids of 3 items in flight; prev row
     L.off_items = o; o += 4 * 32;                       // descriptors of the items n .. n + 3 of this CTA
     L.off_tiles = o; o += nw * L.warp_tile_bytes;
@@ -102,7 +103,7 @@ dq_attn_prepare_kernel(AttnParams p) {
         const int b = head / p.Hq, hq = head % p.Hq, h = hq / p.G, g = hq % p.G;
         if (win < 0) {
             *reinterpret_cast<float4*>(p.qrot + (size_t)head * kN + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
-            uint16_t* rows = p.q16 + ((size_t)b * p.Hkv + h) * 16 * kN;
+            uint16_t* rows = p.q16 + ((size_t)b * p.Hkv + h) * 2 * p.rows * kN;
             __half hi[4], lo[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -115,11 +116,11 @@ dq_attn_prepare_kernel(AttnParams p) {
             *reinterpret_cast<uint2*>(rows + (size_t)g * kN + 4 * lane) = w;
             w.x = (uint32_t)__half_as_ushort(lo[0]) | ((uint32_t)__half_as_ushort(lo[1]) << 16);
             w.y = (uint32_t)__half_as_ushort(lo[2]) | ((uint32_t)__half_as_ushort(lo[3]) << 16);
-            *reinterpret_cast<uint2*>(rows + (size_t)(8 + g) * kN + 4 * lane) = w;
+            *reinterpret_cast<uint2*>(rows + (size_t)(p.rows + g) * kN + 4 * lane) = w;
             if (g == 0)  // unused operand rows of this KV head are zero
-                for (int r = p.G; r < 8; ++r) {
+                for (int r = p.G; r < p.rows; ++r) {
                     *reinterpret_cast<uint2*>(rows + (size_t)r * kN + 4 * lane) = make_uint2(0u, 0u);
-                    *reinterpret_cast<uint2*>(rows + (size_t)(8 + r) * kN + 4 * lane) = make_uint2(0u, 0u);
+                    *reinterpret_cast<uint2*>(rows + (size_t)(p.rows + r) * kN + 4 * lane) = make_uint2(0u, 0u);
                 }
             float s = (v[0] + v[1]) + (v[2] + v[3]);
 #pragma unroll
@@ -262,11 +263,11 @@ __device__ __forceinline__ void decode16_pairs(uint32_t& x, uint32_t& ptr, uint3
 // DO_V the V streams of the previous item are decoded and each finished 16-channel tile of
 // O[j][g] = sum_t (a_t s_t) level_tj (Eq. fold-value, first sum) goes to this warp's output
 // slot in shared memory.  Both decodes are interleaved in one instruction stream.
-template <bool DO_K, bool DO_V, int LBITS, bool PAIRS>
+template <bool DO_K, bool DO_V, int LBITS, bool PAIRS, int ROWS>
 __device__ __forceinline__ void fused_pass(uint32_t xk, uint32_t ptrk, uint32_t xv, uint32_t ptrv, uint32_t lutk,
                                            uint32_t lutv, uint32_t one, uint32_t ktile, uint32_t vtile, uint32_t q16,
                                            uint32_t obuf, int lane, int G, float (&sacc)[4][4],
-                                           const uint32_t (&pb_hi)[2][2], const uint32_t (&pb_lo)[2][2]) {
+                                           const uint32_t (&pb_hi)[ROWS / 8][2][2], const uint32_t (&pb_lo)[ROWS / 8][2][2]) {
     const uint32_t a_addr = q16 + ((lane & 7) + ((lane >> 3) & 1) * 8) * kQ16Stride + (lane >> 4) * 16;
     const int lrow = (lane & 7) + (lane >> 4) * 8;
     const uint32_t ld_off = lrow * 32 + ((((lane >> 3) & 1) ^ ((lrow >> 2) & 1)) << 4);
@@ -294,19 +295,29 @@ __device__ __forceinline__ void fused_pass(uint32_t xk, uint32_t ptrk, uint32_t 
             mma_f16_16816(sacc[1], a, b0[2], b0[3]);
             mma_f16_16816(sacc[2], a, b1[0], b1[1]);
             mma_f16_16816(sacc[3], a, b1[2], b1[3]);
+            if (ROWS == 16) {   // the tile above held q'_hi of all 16 rows; q'_lo adds to the same sums
+                ldmatrix_x4(a, a_addr + kQ16Bytes + cg * 32);
+                mma_f16_16816(sacc[0], a, b0[0], b0[1]);
+                mma_f16_16816(sacc[1], a, b0[2], b0[3]);
+                mma_f16_16816(sacc[2], a, b1[0], b1[1]);
+                mma_f16_16816(sacc[3], a, b1[2], b1[3]);
+            }
         }
         if (DO_V) {
             uint32_t a0[4], a1[4];
-            float o[4] = {0.f, 0.f, 0.f, 0.f};
             ldmatrix_x4_trans(a0, av_addr);                      // tokens 0..15, 16 channels
             ldmatrix_x4_trans(a1, av_addr + 16 * kTileStride);   // tokens 16..31
-            mma_f16_16816(o, a0, pb_hi[0][0], pb_hi[0][1]);
-            mma_f16_16816(o, a1, pb_hi[1][0], pb_hi[1][1]);
-            mma_f16_16816(o, a0, pb_lo[0][0], pb_lo[0][1]);
-            mma_f16_16816(o, a1, pb_lo[1][0], pb_lo[1][1]);
-            const uint32_t oa = o_addr + cg * 64;
-            if (2 * (lane & 3) < G) { sts32f(oa, o[0]); sts32f(oa + 32, o[2]); }
-            if (2 * (lane & 3) + 1 < G) { sts32f(oa + kORow * 4, o[1]); sts32f(oa + kORow * 4 + 32, o[3]); }
+#pragma unroll
+            for (int t = 0; t < ROWS / 8; ++t) {                 // rows 8 t .. 8 t + 7
+                float o[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_f16_16816(o, a0, pb_hi[t][0][0], pb_hi[t][0][1]);
+                mma_f16_16816(o, a1, pb_hi[t][1][0], pb_hi[t][1][1]);
+                mma_f16_16816(o, a0, pb_lo[t][0][0], pb_lo[t][0][1]);
+                mma_f16_16816(o, a1, pb_lo[t][1][0], pb_lo[t][1][1]);
+                const uint32_t oa = o_addr + cg * 64 + t * 8 * kORow * 4;
+                if (8 * t + 2 * (lane & 3) < G) { sts32f(oa, o[0]); sts32f(oa + 32, o[2]); }
+                if (8 * t + 2 * (lane & 3) + 1 < G) { sts32f(oa + kORow * 4, o[1]); sts32f(oa + kORow * 4 + 32, o[3]); }
+            }
         }
         __syncwarp();
     }
@@ -324,15 +335,20 @@ __device__ __forceinline__ void fused_pass(uint32_t xk, uint32_t ptrk, uint32_t 
 // which is how the tests run that path.
 static int step_poll_limit() { return dq_opt_step_poll_limit(DQ_STEP_POLL_LIMIT); }
 // PAIRS: the tables' rANS symbols are pairs of levels (64 steps per stream instead of 128).
-template <bool FUSED, int LBITS, bool PAIRS>
-__global__ void __launch_bounds__(kMaxWarps * 32, 1)
+// ROWS: query rows of a KV head held at once.  16 (several query tokens) takes twice the contractions per decoded
+// level, which is little beside the decode, and eight warps instead of 16 for its output slots; a second pass over
+// the cache would cost the whole decode again.  Four query tokens, 8 sequences of 6016 tokens, 32 / 8 heads: 121.5 us
+// in two passes, 85.0 in one.
+template <bool FUSED, int LBITS, bool PAIRS, int ROWS>
+__global__ void __launch_bounds__((ROWS == 16 ? kRowWarps16 : kMaxWarps) * 32, 1)
 dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant__ DqDevTable TV,
                     const AttnParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nthreads = blockDim.x, nw = nthreads >> 5;
     const int G = p.G;
-    const Layout L = make_layout(nw, TK.rec, TV.rec, p.B, G);
+    const Layout L = make_layout(nw, TK.rec, TV.rec, p.B, G, ROWS);
+    constexpr int kOperand = 2 * ROWS * kQ16Stride;   // bytes of the fp16 q' rows of an item
     const uint32_t sbase = smem_addr(smem);
 
     uint32_t* lutk = reinterpret_cast<uint32_t*>(smem + L.off_lutk);
@@ -341,7 +357,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
     int* s_len = prefix + (p.B + 1);                                // [B] clamped sequence lengths
     float* qsum = reinterpret_cast<float*>(smem + L.off_qsum);      // [2][8]
     float* red_m = reinterpret_cast<float*>(smem + L.off_red);      // [warp][head] chunk maxima
-    float* red_M = red_m + kMaxWarps * DQ_MAX_GROUP;                // [2][head] item maxima
+    float* red_M = red_m + kMaxWarps * ROWS;                        // [2][head] item maxima
     float* obuf_all = reinterpret_cast<float*>(smem + L.off_obuf);  // [warp][head][kORow]
 
     pdl_launch_dependents();
@@ -465,15 +481,15 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                 const uint8_t* s1 = p.k_cont + ((size_t)my_pages[(nk % 3) * 2 + 1] * p.Hkv + ik.h) * blk - blk;
                 for (int i = lane; i < np; i += 32) cp_async16(kst + i * 16, (i < rec ? s0 : s1) + i * 16);
                 if (p.has_mean && lane < G)
-                    cp_async4(kst + L.stage_k - kKTail + lane * 4,
+                    cp_async4(kst + L.stage_k - 4 * ROWS + lane * 4,
                               p.qmu + ((size_t)ik.b * p.Hq + (size_t)ik.h * G + lane) * p.windows + tok0 / DQ_WINDOW_TOKENS);
             }
-            if (tid < 16 * 16) {   // q' operand: 16 rows x 16 pieces of 16 bytes
-                const uint16_t* qsrc = p.q16 + ((size_t)ik.b * p.Hkv + ik.h) * 16 * kN;
-                for (int i = tid; i < 16 * 16; i += nthreads)
-                    cp_async16(sbase + L.off_q16 + (nk & 1) * kQ16Bytes + (i >> 4) * kQ16Stride + (i & 15) * 16, qsrc + i * 8);
+            if (tid < 2 * ROWS * 16) {   // q' operand: 2 ROWS rows x 16 pieces of 16 bytes
+                const uint16_t* qsrc = p.q16 + ((size_t)ik.b * p.Hkv + ik.h) * 2 * ROWS * kN;
+                for (int i = tid; i < 2 * ROWS * 16; i += nthreads)
+                    cp_async16(sbase + L.off_q16 + (nk & 1) * kOperand + (i >> 4) * kQ16Stride + (i & 15) * 16, qsrc + i * 8);
                 if (tid < G)
-                    cp_async4(sbase + L.off_qsum + ((nk & 1) * DQ_MAX_GROUP + tid) * 4,
+                    cp_async4(sbase + L.off_qsum + ((nk & 1) * ROWS + tid) * 4,
                               p.qsum + (size_t)ik.b * p.Hq + (size_t)ik.h * G + tid);
             }
         }
@@ -516,7 +532,11 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
 
     // state carried from the item whose V streams are still to be decoded
     bool have_prev = false;
-    uint32_t pb_hi[2][2] = {{0u, 0u}, {0u, 0u}}, pb_lo[2][2] = {{0u, 0u}, {0u, 0u}};
+    uint32_t pb_hi[ROWS / 8][2][2], pb_lo[ROWS / 8][2][2];
+#pragma unroll
+    for (int t = 0; t < ROWS / 8; ++t)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) { pb_hi[t][i][0] = pb_hi[t][i][1] = pb_lo[t][i][0] = pb_lo[t][i][1] = 0u; }
 
     for (int n = 0;; ++n) {
         Item cur = s_items[n & 3];
@@ -548,7 +568,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
         const uint32_t vst_prev = sbase + L.off_vst + (((n + 1) & 1) * nw + warp) * L.stage_v;
         uint32_t rk = kst + lane * TK.rec;
         const uint32_t rvp = vst_prev + lane * TV.rec;
-        const uint32_t q16 = sbase + L.off_q16 + (n & 1) * kQ16Bytes;
+        const uint32_t q16 = sbase + L.off_q16 + (n & 1) * kOperand;
         float sacc[4][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) { sacc[i][0] = sacc[i][1] = sacc[i][2] = sacc[i][3] = 0.f; }
@@ -558,13 +578,13 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
             constexpr uint32_t kPay = LBITS == 23 ? 8u : 7u;
             const uint32_t xk = lds32_unaligned(rk + 4) & kStateMask, xv = lds32_unaligned(rvp + 4) & kStateMask;
             if (cur.valid && have_prev)
-                fused_pass<true, true, LBITS, PAIRS>(xk, rk + kPay, xv, rvp + kPay, my_lutk, my_lutv, one, ktile, vtile, q16, my_obuf,
+                fused_pass<true, true, LBITS, PAIRS, ROWS>(xk, rk + kPay, xv, rvp + kPay, my_lutk, my_lutv, one, ktile, vtile, q16, my_obuf,
                                               lane, G, sacc, pb_hi, pb_lo);
             else if (cur.valid)
-                fused_pass<true, false, LBITS, PAIRS>(xk, rk + kPay, xv, rvp + kPay, my_lutk, my_lutv, one, ktile, vtile, q16, my_obuf,
+                fused_pass<true, false, LBITS, PAIRS, ROWS>(xk, rk + kPay, xv, rvp + kPay, my_lutk, my_lutv, one, ktile, vtile, q16, my_obuf,
                                                lane, G, sacc, pb_hi, pb_lo);
             else
-                fused_pass<false, true, LBITS, PAIRS>(xk, rk + kPay, xv, rvp + kPay, my_lutk, my_lutv, one, ktile, vtile, q16, my_obuf,
+                fused_pass<false, true, LBITS, PAIRS, ROWS>(xk, rk + kPay, xv, rvp + kPay, my_lutk, my_lutv, one, ktile, vtile, q16, my_obuf,
                                                lane, G, sacc, pb_hi, pb_lo);
         }
 
@@ -573,7 +593,8 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
         tok0 = (cur.blk * nw + warp) * kChunk;
         kst = sbase + L.off_kst + ((n & 1) * nw + warp) * L.stage_k;
         rk = kst + lane * TK.rec;
-        float lg[4][2], sv_t[4][2], ov_t[4][2];
+        constexpr int kSets = ROWS / 8;   // this thread's rows: g_row, and g_row + 8 of 16
+        float lg[kSets][4][2], sv_t[4][2], ov_t[4][2];   // (sv, ov of a token that only the second row sees are kept too)
         if (cur.valid) {
             cp_async_wait<0>();   // the V records of `cur` (header needed now) have landed
             __syncwarp();
@@ -588,19 +609,30 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                 asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};\n" ::"r"(ktile + lane * 16),
                              "f"(sK * p.scale_log2), "f"(oK), "f"(sV), "f"(oV) : "memory");
             }
-            // tokens this thread's row may see: a query token that is not the last one stops earlier; tokens
+            // tokens a row may see: a query token that is not the last one stops earlier; tokens
             // of a BF16 residual window come after the compressed ones and absorb the offset first
-            int row_len = cur.len;
-            if (p.q_total > 1) row_len -= max(0, row_offset(p, g_row) - (p.resid_lens ? max(p.resid_lens[cur.b], 0) : 0));
-            float qmu = 0.f, qs = 0.f;   // q' . window mean and sum of q' (both times the logit scale), for this thread's head row
-            if (g_row < G) {
-                qs = qsum[(n & 1) * DQ_MAX_GROUP + g_row] * p.scale_log2;
-                if (p.has_mean && tok0 < cur.len) qmu = __uint_as_float(lds32(kst + L.stage_k - kKTail + g_row * 4)) * p.scale_log2;
+            int row_len[kSets], most = 0, least = cur.len;
+            float qmu[kSets], qs[kSets];   // q' . window mean and sum of q' (both times the logit scale)
+#pragma unroll
+            for (int t = 0; t < kSets; ++t) {
+                const int row = g_row + 8 * t;
+                row_len[t] = cur.len;
+                if (p.q_total > 1) row_len[t] -= max(0, row_offset(p, row) - (p.resid_lens ? max(p.resid_lens[cur.b], 0) : 0));
+                most = max(most, row_len[t]);
+                least = min(least, row_len[t]);
+                qmu[t] = qs[t] = 0.f;
+                if (row < G) {
+                    qs[t] = qsum[(n & 1) * ROWS + row] * p.scale_log2;
+                    if (p.has_mean && tok0 < cur.len) qmu[t] = __uint_as_float(lds32(kst + L.stage_k - 4 * ROWS + row * 4)) * p.scale_log2;
+                }
             }
             __syncwarp();
-            float mx = -INFINITY;
+            float mx[kSets];
+#pragma unroll
+            for (int t = 0; t < kSets; ++t) mx[t] = -INFINITY;
             const uint32_t meta = ktile + 2 * qd * 16;
-            if (tok0 + kChunk <= row_len) {   // every token of the chunk is visible: no masks
+            const int lim = most - tok0 - 2 * qd;   // token 8 i + 2 qd + u is visible to some row iff 8 i + u < lim
+            auto logits = [&](bool whole) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -608,30 +640,26 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                         float4 m4;
                         asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];\n"
                                      : "=f"(m4.x), "=f"(m4.y), "=f"(m4.z), "=f"(m4.w) : "r"(meta + (8 * i + u) * 16));
-                        lg[i][u] = fmaf(m4.x, sacc[i][u] + sacc[i][2 + u], fmaf(m4.y, qs, qmu));
-                        sv_t[i][u] = m4.z;
-                        ov_t[i][u] = m4.w;
-                        mx = fmaxf(mx, lg[i][u]);
-                    }
-            } else {
-                const int lim = row_len - tok0 - 2 * qd;   // token 8 i + 2 qd + u is visible iff 8 i + u < lim
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        float4 m4;
-                        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-                                     : "=f"(m4.x), "=f"(m4.y), "=f"(m4.z), "=f"(m4.w) : "r"(meta + (8 * i + u) * 16));
-                        const bool ok = 8 * i + u < lim;
-                        lg[i][u] = ok ? fmaf(m4.x, sacc[i][u] + sacc[i][2 + u], fmaf(m4.y, qs, qmu)) : -INFINITY;
+                        const bool ok = whole || 8 * i + u < lim;
                         sv_t[i][u] = ok ? m4.z : 0.f;
                         ov_t[i][u] = ok ? m4.w : 0.f;
-                        mx = fmaxf(mx, lg[i][u]);
+#pragma unroll
+                        for (int t = 0; t < kSets; ++t) {
+                            const float dot = ROWS == 16 ? sacc[i][2 * t + u] : sacc[i][u] + sacc[i][2 + u];
+                            const bool seen = whole || 8 * i + u < row_len[t] - tok0 - 2 * qd;
+                            lg[t][i][u] = seen ? fmaf(m4.x, dot, fmaf(m4.y, qs[t], qmu[t])) : -INFINITY;
+                            mx[t] = fmaxf(mx[t], lg[t][i][u]);
+                        }
                     }
+            };
+            if (tok0 + kChunk <= least) logits(true);   // every token of the chunk is visible: no masks
+            else logits(false);
+#pragma unroll
+            for (int t = 0; t < kSets; ++t) {
+                mx[t] = fmaxf(mx[t], __shfl_xor_sync(kFullMask, mx[t], 1));
+                mx[t] = fmaxf(mx[t], __shfl_xor_sync(kFullMask, mx[t], 2));
+                if (qd == 0) red_m[warp * ROWS + g_row + 8 * t] = mx[t];
             }
-            mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(kFullMask, mx, 2));
-            if (qd == 0) red_m[warp * DQ_MAX_GROUP + g_row] = mx;
         }
         __syncthreads();   // output slots of `prev` complete; chunk maxima of `cur` published
 
@@ -658,7 +686,7 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
                     for (int w = 0; w < nw; ++w) acc += src[w * wstride];
                     float* dst = p.partial + ((size_t)s_prev_row[par] + g) * kPartial;
                     dst[kN + 1 + which] = acc;                   // l at 129, off at 130
-                    if (which == 0) dst[kN] = red_M[par * DQ_MAX_GROUP + g];
+                    if (which == 0) dst[kN] = red_M[par * ROWS + g];
                 }
             }
         }
@@ -666,36 +694,40 @@ dq_attention_kernel(const __grid_constant__ DqDevTable TK, const __grid_constant
         // ------------------------------------------ softmax weights of `cur`, scaled by the item maximum
         have_prev = cur.valid;
         if (cur.valid) {
-            float m_item = -INFINITY;   // the four threads of a head row share the warps' maxima
-            for (int w = qd; w < nw; w += 4) m_item = fmaxf(m_item, red_m[w * DQ_MAX_GROUP + g_row]);
-            m_item = fmaxf(m_item, __shfl_xor_sync(kFullMask, m_item, 1));
-            m_item = fmaxf(m_item, __shfl_xor_sync(kFullMask, m_item, 2));
-            if (warp == 0 && qd == 0) red_M[(n & 1) * DQ_MAX_GROUP + g_row] = m_item;
-            const float m_use = (m_item == -INFINITY) ? 0.f : m_item;
-            float lsum = 0.f, osum = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float ps[2];
+            for (int t = 0; t < kSets; ++t) {
+                const int row = g_row + 8 * t;
+                float m_item = -INFINITY;   // the four threads of a row share the warps' maxima
+                for (int w = qd; w < nw; w += 4) m_item = fmaxf(m_item, red_m[w * ROWS + row]);
+                m_item = fmaxf(m_item, __shfl_xor_sync(kFullMask, m_item, 1));
+                m_item = fmaxf(m_item, __shfl_xor_sync(kFullMask, m_item, 2));
+                if (warp == 0 && qd == 0) red_M[(n & 1) * ROWS + row] = m_item;
+                const float m_use = (m_item == -INFINITY) ? 0.f : m_item;
+                float lsum = 0.f, osum = 0.f;
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const float pr = ex2_approx(lg[i][u] - m_use);   // <= 1; exp2(-inf) = 0
-                    lsum += pr;
-                    osum = fmaf(pr, ov_t[i][u], osum);
-                    ps[u] = pr * sv_t[i][u];
+                for (int i = 0; i < 4; ++i) {
+                    float ps[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const float pr = ex2_approx(lg[t][i][u] - m_use);   // <= 1; exp2(-inf) = 0
+                        lsum += pr;
+                        osum = fmaf(pr, ov_t[i][u], osum);
+                        ps[u] = pr * sv_t[i][u];
+                    }
+                    // fp16 hi + lo pair of each weight: hi = rn(ps), lo = rn(ps - hi)
+                    const __half2 h2 = __floats2half2_rn(ps[0], ps[1]);
+                    const float2 hf = __half22float2(h2);
+                    pb_hi[t][i >> 1][i & 1] = *reinterpret_cast<const uint32_t*>(&h2);
+                    pb_lo[t][i >> 1][i & 1] = pack_half2(ps[0] - hf.x, ps[1] - hf.y);
                 }
-                // fp16 hi + lo pair of each weight: hi = rn(ps), lo = rn(ps - hi)
-                const __half2 h2 = __floats2half2_rn(ps[0], ps[1]);
-                const float2 hf = __half22float2(h2);
-                pb_hi[i >> 1][i & 1] = *reinterpret_cast<const uint32_t*>(&h2);
-                pb_lo[i >> 1][i & 1] = pack_half2(ps[0] - hf.x, ps[1] - hf.y);
-            }
-            lsum += __shfl_xor_sync(kFullMask, lsum, 1);
-            lsum += __shfl_xor_sync(kFullMask, lsum, 2);
-            osum += __shfl_xor_sync(kFullMask, osum, 1);
-            osum += __shfl_xor_sync(kFullMask, osum, 2);
-            if (qd == 0 && g_row < G) {   // l and off ride along in this warp's output slot (columns by parity)
-                sts32f(my_obuf + (g_row * kORow + kN + 2 * (n & 1)) * 4, lsum);
-                sts32f(my_obuf + (g_row * kORow + kN + 2 * (n & 1) + 1) * 4, osum);
+                lsum += __shfl_xor_sync(kFullMask, lsum, 1);
+                lsum += __shfl_xor_sync(kFullMask, lsum, 2);
+                osum += __shfl_xor_sync(kFullMask, osum, 1);
+                osum += __shfl_xor_sync(kFullMask, osum, 2);
+                if (qd == 0 && row < G) {   // l and off ride along in this warp's output slot (columns by parity)
+                    sts32f(my_obuf + (row * kORow + kN + 2 * (n & 1)) * 4, lsum);
+                    sts32f(my_obuf + (row * kORow + kN + 2 * (n & 1) + 1) * 4, osum);
+                }
             }
         }
         if (tid == 0) s_prev_row[n & 1] = (long long)cur.bg * p.Hq + (long long)cur.h * G;   // read after two barriers
@@ -1066,17 +1098,19 @@ inline int windows_for(int max_pages) {
     return (max_pages * DQ_PAGE_TOKENS + DQ_WINDOW_TOKENS - 1) / DQ_WINDOW_TOKENS;
 }
 
-WsLayout ws_layout(int B, int Hq, int max_pages) {
+// rows: query rows a KV head's operand holds (0: the 8-row layout for any Hkv <= Hq, what callers allocate); min_item:
+// fewest tokens an item may have
+WsLayout ws_layout(int B, int Hq, int max_pages, int Hkv = 0, int rows = 0, int min_item = kMinItemTokens) {
     WsLayout w;
     size_t o = 0;
     auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
     w.off_counter = o; o += 16;
     w.off_prefix = o; o += up((size_t)(B + 1) * 8);   // block prefix sums, then non-empty-sequence counts
     w.off_qrot = o; o += (size_t)B * Hq * kN * 4;
-    w.off_q16 = o; o += (size_t)B * Hq * 16 * kN * 2;   // Hkv <= Hq rows blocks
+    w.off_q16 = o; o += rows ? (size_t)B * Hkv * 2 * rows * kN * 2 : (size_t)B * Hq * 16 * kN * 2;   // Hkv <= Hq rows blocks
     w.off_qsum = o; o += up((size_t)B * Hq * 4);
     w.off_qmu = o; o += up((size_t)B * Hq * windows_for(max_pages) * 4);
-    const size_t blocks = (size_t)B * (((size_t)max_pages * DQ_PAGE_TOKENS + kMinItemTokens - 1) / kMinItemTokens);
+    const size_t blocks = (size_t)B * (((size_t)max_pages * DQ_PAGE_TOKENS + min_item - 1) / min_item);
     w.off_partial = o; o += blocks * Hq * kPartial * 4;
     w.total = o;
     return w;
@@ -1138,28 +1172,28 @@ static cudaError_t device_limits(int* sm_count, int* smem_max) {
     return cudaSuccess;
 }
 
-// One pass: query tokens [q_first, q_first + q_len) of the q_total given; q_len * (Hq / Hkv) <= 8.
+// One pass: query tokens [q_first, q_first + q_len) of the q_total given; q_len * (Hq / Hkv) <= rows (8 or 16).
 static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable& tv, const DqAttnArgs& a, int q_total,
-                                         int q_first, int q_len, cudaStream_t st) {
+                                         int q_first, int q_len, int rows, cudaStream_t st) {
     int sm_count = 0, smem_max = 0;
     {
         const cudaError_t e = device_limits(&sm_count, &smem_max);
         if (e != cudaSuccess) return e;
     }
-    int nw = kMaxWarps;
+    int nw = rows == 16 ? kRowWarps16 : kMaxWarps;
     const int G1 = a.Hq / a.Hkv, G = G1 * q_len;   // rows per KV head
     const bool wide = tk.hs > 1;   // token-wide streams: main kernel of dq_attention_wide.cu
-    Layout L = make_layout(nw, tk.rec, tv.rec, a.B, G);
-    const int small = dq_attn_small_pick_warps(tk, tv, a.B, a.Hkv, a.max_pages, sm_count, smem_max);
+    Layout L = make_layout(nw, tk.rec, tv.rec, a.B, G, rows);
+    const int small = rows == 16 ? 0 : dq_attn_small_pick_warps(tk, tv, a.B, a.Hkv, a.max_pages, sm_count, smem_max);
     if (small) {
         nw = small;
     } else if (wide) {
         nw = dq_attn_wide_pick_warps(tk, tv, a.B, G, a.Hkv / tk.hs, a.max_pages, sm_count, smem_max);
         if (nw == 0) return cudaErrorInvalidConfiguration;
     } else {
-        while (L.total > smem_max && nw > 4) {
+        while (L.total > smem_max && nw > (rows == 16 ? kRowWarps16 : 4)) {
             nw -= 2;
-            L = make_layout(nw, tk.rec, tv.rec, a.B, G);
+            L = make_layout(nw, tk.rec, tv.rec, a.B, G, rows);
         }
         // A CTA makes one pass more than it has blocks, and a pass takes about 7.5 + 0.33 nw us: fewer warps where that
         // saves the last, nearly empty round (blocks counted from the width of the page table).
@@ -1168,18 +1202,20 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
             return ((blocks + sm_count - 1) / sm_count + 1) * (7.5 + 0.33 * w);
         };
         int best = nw;
-        for (int w = nw - 2; w >= 8; w -= 2)
+        for (int w = nw - 2; w >= 8 && rows == 8; w -= 2)
             if (cost(w) < cost(best)) best = w;
         if (best != nw) {
             nw = best;
-            L = make_layout(nw, tk.rec, tv.rec, a.B, G);
+            L = make_layout(nw, tk.rec, tv.rec, a.B, G, rows);
         }
         if (L.total > smem_max) return cudaErrorInvalidConfiguration;
     }
 
-    const WsLayout w = ws_layout(a.B, a.Hq * q_len, a.max_pages);
+    const WsLayout w = rows == 16 ? ws_layout(a.B, a.Hq * q_len, a.max_pages, a.Hkv, 16, kRowWarps16 * kChunk)
+                                  : ws_layout(a.B, a.Hq * q_len, a.max_pages);
     uint8_t* ws = static_cast<uint8_t*>(a.workspace);
     AttnParams p;
+    p.rows = rows;
     p.q = static_cast<const uint16_t*>(a.q_bf16);
     p.k_cont = a.k_cont; p.v_cont = a.v_cont;
     p.mean_q = a.mean_q; p.mean_scale = a.mean_scale;
@@ -1231,10 +1267,12 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
     if (e != cudaSuccess) return e;
     // the four instantiations of the main kernel: decode-step mode or not, 32- or 24-bit final state
     void (*main_kernel)(DqDevTable, DqDevTable, AttnParams) =
-        tk.pair ? (tk.sigma == 24 ? (p.fused ? dq_attention_kernel<true, 15, true> : dq_attention_kernel<false, 15, true>)
-                                  : (p.fused ? dq_attention_kernel<true, 23, true> : dq_attention_kernel<false, 23, true>))
-                : (tk.sigma == 24 ? (p.fused ? dq_attention_kernel<true, 15, false> : dq_attention_kernel<false, 15, false>)
-                                  : (p.fused ? dq_attention_kernel<true, 23, false> : dq_attention_kernel<false, 23, false>));
+        rows == 16 ? (tk.pair ? (tk.sigma == 24 ? dq_attention_kernel<false, 15, true, 16> : dq_attention_kernel<false, 23, true, 16>)
+                              : (tk.sigma == 24 ? dq_attention_kernel<false, 15, false, 16> : dq_attention_kernel<false, 23, false, 16>))
+        : tk.pair ? (tk.sigma == 24 ? (p.fused ? dq_attention_kernel<true, 15, true, 8> : dq_attention_kernel<false, 15, true, 8>)
+                                    : (p.fused ? dq_attention_kernel<true, 23, true, 8> : dq_attention_kernel<false, 23, true, 8>))
+                  : (tk.sigma == 24 ? (p.fused ? dq_attention_kernel<true, 15, false, 8> : dq_attention_kernel<false, 15, false, 8>)
+                                    : (p.fused ? dq_attention_kernel<true, 23, false, 8> : dq_attention_kernel<false, 23, false, 8>));
     if (!wide) {
         e = dq_allow_smem(reinterpret_cast<const void*>(main_kernel), L.total);
         if (e != cudaSuccess) return e;
@@ -1248,14 +1286,28 @@ static cudaError_t launch_attention_pass(const DqDevTable& tk, const DqDevTable&
 }
 
 // q_len query tokens per sequence: as many passes over the cache as it takes to give every
-// (query token, head) pair of a KV head one of the 8 rows of the MMA tile.
+// (query token, head) pair of a KV head one of the 8 or 16 rows of the MMA tile.
 cudaError_t dq_launch_attention(const DqDevTable& tk, const DqDevTable& tv, const DqAttnArgs& a,
                                 cudaStream_t st) {
-    const int q_total = a.q_len > 1 ? a.q_len : 1;
-    const int per_pass = DQ_MAX_GROUP / (a.Hq / a.Hkv) > 0 ? DQ_MAX_GROUP / (a.Hq / a.Hkv) : 1;
+    const int q_total = a.q_len > 1 ? a.q_len : 1, G1 = a.Hq / a.Hkv;
+    int rows = 8, per_pass = DQ_MAX_GROUP / G1 > 0 ? DQ_MAX_GROUP / G1 : 1;
+    if (q_total > per_pass && tk.hs == 1 && !a.fused) {
+        // More rows than one tile: 16 at a time where that saves a pass, their scratch fits what the caller gave (sized
+        // for eight) and the shared memory holds eight warps.  Saves a pass of the single-wave kernel too: two of those
+        // take 29 us at Hq / Hkv = 32 / 8 and 200 to 4000 tokens, one pass of 16 rows 22 us.
+        int sm_count = 0, smem_max = 0;
+        const cudaError_t e = device_limits(&sm_count, &smem_max);
+        if (e != cudaSuccess) return e;
+        int per16 = q_total < 16 / G1 ? q_total : 16 / G1;
+        while (per16 > per_pass && (ws_layout(a.B, a.Hq * per16, a.max_pages, a.Hkv, 16, kRowWarps16 * kChunk).total > a.workspace_bytes ||
+                                    make_layout(kRowWarps16, tk.rec, tv.rec, a.B, G1 * per16, 16).total > smem_max))
+            --per16;
+        const int passes8 = (q_total + per_pass - 1) / per_pass, passes16 = (q_total + per16 - 1) / per16;
+        if (passes16 < passes8) { rows = 16; per_pass = per16; }
+    }
     for (int q_first = 0; q_first < q_total; q_first += per_pass) {
         const int q_len = q_total - q_first < per_pass ? q_total - q_first : per_pass;
-        const cudaError_t e = launch_attention_pass(tk, tv, a, q_total, q_first, q_len, st);
+        const cudaError_t e = launch_attention_pass(tk, tv, a, q_total, q_first, q_len, q_len * G1 > 8 ? rows : 8, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1296,7 +1348,7 @@ cudaError_t dq_launch_bf16_attention(const DqAttnArgs& a, const void* k_pages, c
     p.scale_log2 = a.sm_scale * 1.4426950408889634f;
     p.hkv_magic = 0;
     p.hs = 1; p.groups = a.Hkv;
-    p.q_len = 1; p.G1 = p.G; p.Hq1 = a.Hq; p.q_total = 1; p.q_first = 0;
+    p.q_len = 1; p.G1 = p.G; p.Hq1 = a.Hq; p.q_total = 1; p.q_first = 0; p.rows = 8;
     p.fused = 0; p.attn_grid = 0; p.poll_limit = 0; p.flags = p.counter; p.ne_before = p.prefix + (a.B + 1);
     p.resid_k = nullptr; p.resid_v = nullptr; p.resid_lens = nullptr; p.resid_cap = 0;
     const int heads = a.B * a.Hq;

@@ -28,7 +28,7 @@ struct AttnParams {
     int* counter;
     int* prefix;        // [B + 1] blocks before sequence b
     float* qrot;        // [B][Hq][128]              rotated q (bf16 baseline reads q itself)
-    uint16_t* q16;      // [B][Hkv][16][128] halves  fp16 hi (rows g) / lo (rows 8 + g) of q'
+    uint16_t* q16;      // [B][Hkv][2 rows][128] halves  fp16 hi (rows g) / lo (rows `rows` + g) of q'
     float* qsum;        // [B][Hq]                   sum_j q'_j
     float* qmu;         // [B][Hq][windows]          sum_j q'_j mean_j of every window
     float* partial;     // [blocks][Hq][kPartial]
@@ -41,6 +41,7 @@ struct AttnParams {
     // Several query tokens per sequence (q_len > 1): the rows of one KV head are (query token i, head g),
     // r = i * G1 + g; G = q_len * G1 rows per KV head and Hq = Hkv * G rows per sequence everywhere in the
     // workspace.  Query token i is q_len - 1 - i positions before the end of the sequence.
+    int rows;           // query rows of a KV head that the operand holds: 8, or 16 (hi rows first, then lo rows)
     int q_len, G1, Hq1; // query tokens of this pass; query heads per KV head and per token
     // Decode-step mode (dq_decode_step): the attention kernel starts while the step's encoder still runs.
     // flags: [0] next dynamic item, [1] set when the prepare kernel's outputs are complete, [2] prepare

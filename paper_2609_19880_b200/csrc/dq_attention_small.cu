@@ -6,7 +6,6 @@
 //     for the softmax weights, so a block costs one pass over the streams instead of two;
 //   * no prepare kernel: a CTA rotates its own q rows, takes q'.mean of its windows and scans the sequence lengths;
 //   * decode-step mode: only the CTAs whose block holds a sequence's newest token wait for the encoder.
-// Compiled with ptxas -O1, which keeps the interleaved order (at -O3 the scheduler puts one chain after the other).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 

@@ -111,6 +111,7 @@ struct DqAttnArgs {
     const int32_t* resid_lens;  // [B]
     int resid_cap;
     int q_len;                  // query tokens per sequence (q and out are [B][q_len][Hq][128]); 0 or 1: one
+    size_t workspace_bytes;     // 0: no more than the 8-row layout needs
     int fused;                  // decode-step mode: launched right after the step's encoder (see dq_decode_step)
 };
 size_t dq_attn_workspace_bytes(int B, int Hq, int max_pages);
