@@ -349,11 +349,12 @@ static __device__ __noinline__ uint2 drift_pair_search(const EncTable& T, float 
     return make_uint2(len, (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24));
 }
 
-// Levels of the nearest pairs when they fit the budget (every test of the bisection then passes and lambda ends too
-// small to move any pair) and no value is within rounding of a midpoint.
+// Levels of the nearest pairs: Drift's outcome when their length, summed over the stream, fits the budget (every test of the
+// bisection then passes and lambda ends too small to move any pair) and no `clear` of the stream is negative (no value
+// within rounding of a midpoint).  False where the bound on rounding does not hold.
 template <int M>
-__device__ __forceinline__ bool drift_pair_nearest(const EncTable& T, const float (&z)[4], float s, float o, float zmin, float zmax,
-                                                   uint32_t& sym) {
+__device__ __forceinline__ bool nearest_pairs(const EncTable& T, const float (&z)[4], float s, float o, float zmin, float zmax,
+                                              uint32_t& sym, uint32_t& len, float& clear) {
     if (!(s > 0x1p-30f && s < 0x1p40f)) return false;
     const float inv = dqdrift::rcp_approx(s), shift = -o * inv;
     const float vmax = fmaf(zmax, inv, shift), vmin = fmaf(zmin, inv, shift);
@@ -369,16 +370,21 @@ __device__ __forceinline__ bool drift_pair_nearest(const EncTable& T, const floa
         mid = fminf(mid, fabsf(fabsf(v - near[e]) - 0.5f));
     }
     const uint32_t u0 = (uint32_t)(int)fmaf(near[0], (float)M, near[1]), u1 = (uint32_t)(int)fmaf(near[2], (float)M, near[3]);
-    const uint32_t len = __reduce_add_sync(kFull, (T.prk[u0].y >> 8) + (T.prk[u1].y >> 8));
+    len = (T.prk[u0].y >> 8) + (T.prk[u1].y >> 8);
     sym = (u0 / M) | ((u0 % M) << 8) | ((u1 / M) << 16) | ((u1 % M) << 24);
-    return len <= ((uint32_t)T.budget_bits << 16) && __all_sync(kFull, mid > E);
+    clear = mid - E;
+    return true;
 }
 
 // Length of the assignment (0: known to be within the budget); sym: its levels, one per byte.
 template <int M>
 __device__ __forceinline__ uint32_t drift_pair(const EncTable& T, const float (&z)[4], float s, float o, float zmin, float zmax,
                                                uint32_t& sym) {
-    if (drift_pair_nearest<M>(T, z, s, o, zmin, zmax, sym)) return 0u;
+    uint32_t len;
+    float clear;
+    if (nearest_pairs<M>(T, z, s, o, zmin, zmax, sym, len, clear) && __reduce_add_sync(kFull, len) <= ((uint32_t)T.budget_bits << 16) &&
+        __all_sync(kFull, clear > 0.f))
+        return 0u;
     const uint2 r = drift_pair_search<M>(T, z[0], z[1], z[2], z[3], s, o);
     sym = r.y;
     return r.x;

@@ -26,11 +26,51 @@ struct WideShared {
     int J;                           // cell that the histogram search ends in
 };
 
+// Smallest difference of two level costs whose code lengths differ.
+template <int M>
+__device__ __forceinline__ float least_cost_step(const float (&rm)[M], const uint32_t (&Km)[M]) {
+    float dr = 1e30f;
+#pragma unroll
+    for (int m = 1; m < M; ++m)
+#pragma unroll
+        for (int n = 0; n < m; ++n)
+            if ((Km[m] ^ Km[n]) >> 8) dr = fminf(dr, fabsf(rm[m] - rm[n]));
+    return dr;
+}
+
+// The bisection's outcome from where it nearly certainly ends: the length at lambda_{J+1} of its 4096-point grid within the
+// budget, the one at lambda_J over it; otherwise J moves by one.  2 sweeps instead of 13: 713 -> 699 us for 5 prompts of
+// 1000 to 4000 tokens (the per-head kernel, short of registers, lost 2 % with it).  sweep(lambda) returns the
+// length and leaves the winners in sym; kept: those at lambda_{J+1}.  Lengths fall with lambda, except where rounding
+// decides: between points closer than 2^-21 of the largest cost over the smallest difference of two r (dr); there, and
+// when J is not found, the result is false.
+template <class Sweep>
+__device__ __forceinline__ bool confirm_cell(const Sweep& sweep, int J, uint32_t budget, float lam_lo0, float lam_hi0, float maxD, float dr,
+                                             const uint32_t (&sym)[4], uint32_t (&kept)[4]) {
+#pragma unroll 1
+    for (int t = 0; t < 3; ++t) {
+        if (J < 1 || J > 4094) return false;
+        float lo = lam_lo0, hi = lam_hi0;
+#pragma unroll 1
+        for (int b = 11; b >= 0; --b) {
+            const float mid = __fsqrt_rn(__fmul_rn(lo, hi));
+            if ((J >> b) & 1) lo = mid; else hi = mid;
+        }
+        if (!(lo * (0.0067f * dr) > 0x1p-21f * (maxD + hi * 8.f))) return false;   // r <= 8
+        if (sweep(hi) > budget) { ++J; continue; }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) kept[e] = sym[e];
+        if (sweep(lo) > budget) return true;
+        --J;
+    }
+    return false;
+}
+
 // Function Drift of Algorithm 1 for a stream held by hs warps; same arithmetic as drift_sweeps, with
 // the extrema of D and the code length taken over the whole stream.
 template <int M>
 __device__ __forceinline__ uint2 drift_wide_sweeps(const EncTable& T, WideShared& W, int hs, int wib, uint32_t& parity,
-                                                   const float (&z)[4], float s, float o) {
+                                                   const float (&z)[4], float s, float o, int cell) {
     const int lane = threadIdx.x & 31;
     float tm[M], rm[M];
     uint32_t Km[M];   // ceil(65536 r_m) << 8 | m: the minimum tree carries one word for length and index
@@ -64,14 +104,7 @@ __device__ __forceinline__ uint2 drift_wide_sweeps(const EncTable& T, WideShared
     float lam_hi = __fmul_rn(8.0f, __fsub_rn(maxD, minD));
     float lam_lo = __fmul_rn(lam_hi, 0x1p-40f);
     uint32_t len = 0, sym[4] = {0u, 0u, 0u, 0u};
-    // Early-exit variant: when each of the 12 tests passes, the upper end walks hi <- sqrt(lo hi) twelve
-    // times with lo fixed; sweep -1 evaluates that multiplier and ends the search if its assignment fits.
-    float lam_e = lam_hi;
-    if (T.early_exit)
-        for (int i = 0; i < 12; ++i) lam_e = __fsqrt_rn(__fmul_rn(lam_lo, lam_e));
-#pragma unroll 1
-    for (int it = T.early_exit ? -1 : 0; it <= 12; ++it) {
-        const float lam = (it < 0) ? lam_e : (it < 12) ? __fsqrt_rn(__fmul_rn(lam_lo, lam_hi)) : lam_hi;
+    auto sweep = [&](float lam) {
         uint32_t cost_sum = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -90,11 +123,25 @@ __device__ __forceinline__ uint2 drift_wide_sweeps(const EncTable& T, WideShared
         const uint32_t wl = __reduce_add_sync(kFull, cost_sum >> 8);
         if (lane == 0) W.len[parity][wib] = wl;
         __syncthreads();
-        len = 0;
-        for (int w = 0; w < hs; ++w) len += W.len[parity][w];
+        uint32_t sum = 0;
+        for (int w = 0; w < hs; ++w) sum += W.len[parity][w];   // every warp sees the same stream-wide length
         parity ^= 1u;
+        return sum;
+    };
+    uint32_t kept[4];
+    if (cell > 0 && confirm_cell(sweep, cell, budget, lam_lo, lam_hi, maxD, least_cost_step<M>(rm, Km), sym, kept))
+        return make_uint2(0u, (kept[0] & 0xffu) | ((kept[1] & 0xffu) << 8) | ((kept[2] & 0xffu) << 16) | (kept[3] << 24));
+    // Early-exit variant: when each of the 12 tests passes, the upper end walks hi <- sqrt(lo hi) twelve
+    // times with lo fixed; sweep -1 evaluates that multiplier and ends the search if its assignment fits.
+    float lam_e = lam_hi;
+    if (T.early_exit)
+        for (int i = 0; i < 12; ++i) lam_e = __fsqrt_rn(__fmul_rn(lam_lo, lam_e));
+#pragma unroll 1
+    for (int it = T.early_exit ? -1 : 0; it <= 12; ++it) {
+        const float lam = (it < 0) ? lam_e : (it < 12) ? __fsqrt_rn(__fmul_rn(lam_lo, lam_hi)) : lam_hi;
+        len = sweep(lam);
         if (it < 0) {
-            if (len <= budget) break;   // uniform across the CTA: every warp sees the same stream-wide length
+            if (len <= budget) break;   // uniform across the CTA
         } else if (it < 12) {
             if (len <= budget) lam_hi = lam; else lam_lo = lam;
         }
@@ -197,12 +244,14 @@ __device__ __forceinline__ float slots_min(const float* slot, int hs) { return d
 // into every grid cell, so J is found by a histogram of the thresholds' cells with a suffix sum over it (the
 // sums and maxima that serve 128 values would each be a CTA barrier here).  A threshold counts for the cell of the
 // lower end of its error interval: the length at lambda_J is then certainly over the budget, and the one at
-// lambda_{J+1} is exact unless some interval holds that point, which is a tie.  Returns false on a tie.
+// lambda_{J+1} is exact unless some interval holds that point, which is a tie.  Returns false on a tie, with the cell J
+// (-1: none) that the sweeps then try first.
 // hist: kCells words, zero on entry and on return.
 template <int M>
 __device__ __forceinline__ bool drift_wide_thresholds(const EncTable& T, WideShared& W, uint32_t* hist, int hs, int wib,
                                                       uint32_t& parity, const float (&z)[4], float s, float o, float zmin,
-                                                      float zmax, uint32_t& sym) {
+                                                      float zmax, uint32_t& sym, int& cell) {
+    cell = -1;
     constexpr int kC = (M - 1) / 2, kLow = kC, kHigh = M - 1 - kC;
     const int lane = threadIdx.x & 31;
     if (!(s > 0x1p-30f && s < 0x1p40f)) return false;
@@ -303,6 +352,7 @@ __device__ __forceinline__ bool drift_wide_thresholds(const EncTable& T, WideSha
         __syncthreads();
         const int J = W.J;
         tie = J < 2 || J > 4092;
+        if (!tie) cell = J;
         yf = dqdrift::exp2_approx(fmaf((float)(J + 1 - 3072), 1.f / 102.4f, lgD));
         // wider than the histogram's intervals, so that an edge whose cell and final comparison disagree is always a tie
         band = fmaf(yf, 1.5f * wA * (1.f / 148.f), 1.5f * band);
@@ -329,9 +379,9 @@ __device__ __forceinline__ bool drift_wide_thresholds(const EncTable& T, WideSha
 // The sweeps of a stream that the thresholds leave open: {length, this lane's four levels}.
 template <int M>
 __device__ __noinline__ uint2 drift_wide_sweeps_m(const EncTable& T, WideShared& W, int hs, int wib, uint32_t parity, float z0, float z1,
-                                                  float z2, float z3, float s, float o) {
+                                                  float z2, float z3, float s, float o, int cell) {
     const float z[4] = {z0, z1, z2, z3};
-    return drift_wide_sweeps<M>(T, W, hs, wib, parity, z, s, o);
+    return drift_wide_sweeps<M>(T, W, hs, wib, parity, z, s, o, cell);
 }
 
 // Drift on the CTA's stream: {length (0: known to be within the budget), this lane's four levels}.
@@ -339,10 +389,23 @@ template <int M, bool PAIR>
 __device__ __forceinline__ uint2 drift_wide(const EncTable& T, WideShared& W, uint32_t* hist, int hs, int wib, uint32_t& parity,
                                             const float (&z)[4], float s, float o, float zmin, float zmax) {
     uint2 r = make_uint2(0u, 0u);
+    int cell;
     if (PAIR) {
+        uint32_t len;
+        float clear;
+        if (nearest_pairs<M>(T, z, s, o, zmin, zmax, r.y, len, clear)) {   // uniform: extrema and grid are stream-wide
+            len = __reduce_add_sync(kFull, len);
+            clear = dqdev::warp_min(clear);
+            if ((threadIdx.x & 31) == 0) { W.len[parity][wib] = len; W.fmin[parity][wib] = clear; }
+            __syncthreads();
+            len = slots_add(W.len[parity], hs);
+            clear = slots_min(W.fmin[parity], hs);
+            parity ^= 1u;
+            if (len <= ((uint32_t)T.budget_bits << 16) && clear > 0.f) return r;
+        }
         r = drift_wide_pairs<M>(T, W, hs, wib, parity, z, s, o);
-    } else if (!drift_wide_thresholds<M>(T, W, hist, hs, wib, parity, z, s, o, zmin, zmax, r.y)) {
-        r = drift_wide_sweeps_m<M>(T, W, hs, wib, parity, z[0], z[1], z[2], z[3], s, o);
+    } else if (!drift_wide_thresholds<M>(T, W, hist, hs, wib, parity, z, s, o, zmin, zmax, r.y, cell)) {
+        r = drift_wide_sweeps_m<M>(T, W, hs, wib, parity, z[0], z[1], z[2], z[3], s, o, cell);
         __syncthreads();   // the slots of either parity are free again
     }
     return r;
