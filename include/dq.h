@@ -171,7 +171,7 @@ int dq_tables_info(const dq_tables *t, dq_table_info *out);
  *                    fell back to the all-central assignment, [1] constant streams,
  *                    [2] rejected refits, [3] max record bytes used (atomicMax).
  * With token-wide tables (heads_per_stream = hs > 1; both tables must agree, Hkv % hs == 0) one
- * CTA of hs warps encodes a stream and the containers use the interleaved layout.
+ * CTA of hs warps encodes one to 32 streams and the containers use the interleaved layout.
  * Calls with many streams (prefill, bulk encodes) run batch kernels that code 32 streams per CTA;
  * the records are the same.  The option DQ_OPT_ENCODE_BATCH_MIN (a stream count, dq_set_option)
  * moves the size from which they are used.
